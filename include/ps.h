@@ -244,9 +244,9 @@ typedef struct {
 
 /* Compile the program's instruction lists into one kernel at creation (NVRTC, sm_103a): the
  * slot file in registers, the byte-code's slots and immediates as constants.  Same results as
- * the interpreter up to the rounding of fused multiply-adds across op boundaries.  Programs of
- * more than six channels are compiled one unit per channel, in parallel on host threads, and
- * linked (nvJitLink) into one kernel.  Creation fails (PS_ERR_GRAPH with the compiler's message,
+ * the interpreter up to the rounding of fused multiply-adds across op boundaries.  FP64
+ * programs of more than two channels, and mixed ones of more than six, are compiled one unit per
+ * channel, in parallel on host threads, and linked (nvJitLink) into one kernel.  Creation fails (PS_ERR_GRAPH with the compiler's message,
  * PS_ERR_CUDA) if the kernel cannot be built.  Compiled kernels (and the split form's channel
  * units) are cached per device and source for the life of the process: a second program with
  * the same channels and options costs no compilation, and the cached modules are never unloaded. */

@@ -30,10 +30,13 @@ using dev::P4;
 
 constexpr int kMaxLeg = kMaxOutMomenta + 2;
 
+// Both inverse maps: where rounding has collapsed the range to a point every r maps to it, and 0 is
+// returned (the quotients below would be 0/0 or infinite).
 // inverse power-law map (anchored as the forward map)
 __device__ __forceinline__ double inv_nu(double x, double m, double nu, double xmin, double xmax, double a) {
     const double m2 = (m > 0.0) ? m * m : -a;
     const double lo = xmin - m2, hi = xmax - m2;
+    if (xmax <= xmin) return 0.0;
     const double L = log1p((xmax - xmin) / lo);
     if (nu == 1.0) return log1p((x - xmin) / lo) / L;
     const double w = 1.0 - nu;
@@ -45,6 +48,7 @@ __device__ __forceinline__ double inv_nu(double x, double m, double nu, double x
 __device__ __forceinline__ double inv_bw(double x, double M, double G, double xmin, double xmax) {
     const double mg = M * G, m2 = M * M;
     const double a = (xmin - m2) / mg, b = (xmax - m2) / mg;
+    if (xmax <= xmin) return 0.0;
     const double D = atan2((xmax - xmin) / mg, fma(a, b, 1.0));
     const double t = (x - m2) / mg;
     if (x - xmin <= xmax - x) return atan2((x - xmin) / mg, fma(a, t, 1.0)) / D;

@@ -22,6 +22,7 @@
 #include <nvrtc.h>
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cinttypes>
 #include <cstdio>
@@ -103,6 +104,36 @@ struct InvariantMemo {
     }
 };
 
+// Slots of output i of an op: a momentum's four, or a scalar's one.
+int out_width(int op, int i) {
+    switch (op) {
+        case PS_OP_TWO_TO_TWO_COM:
+        case PS_OP_TWO_BODY_DECAY:
+        case PS_OP_TWO_BODY_DECAY_COM: return i < 2 ? 4 : 1;
+        case PS_OP_COM_P_IN:
+        case PS_OP_BOOST_BEAM:
+        case PS_OP_MOM_ADD:
+        case PS_OP_MOM_SUB: return 4;
+        default: return 1;
+    }
+}
+
+// The t ranges of a channel by their arguments (slots, or immediates ~i): forgotten when an argument's
+// slot is written.
+struct RangeMemo {
+    std::map<std::array<int32_t, 5>, std::string> names;
+    int next = 0;
+    static bool reads(const std::array<int32_t, 5>& key, int32_t o, int32_t n) {
+        for (int32_t k : key)
+            if (k >= o && k < o + n) return true;
+        return false;
+    }
+    void written(int32_t o, int32_t n) {
+        for (auto it = names.begin(); it != names.end();)
+            it = reads(it->first, o, n) ? names.erase(it) : std::next(it);
+    }
+};
+
 // The SDE weight of another channel (PS_OP_CHANNEL_WEIGHT: k, p_a, q_1..q_k, (kind, mask, M,
 // Gamma)...) as straight-line code: each propagator's invariant from the memo (declared in *decl
 // before the op's block at its first use), the propagator arithmetic from the interpreter's
@@ -154,7 +185,7 @@ std::string channel_weight_source(const Compiled& C, const int32_t* a, int na, b
                  ", " + hexlit(G) + ");\n";
     }
     s += mixed ? "                  dev::st(f, " + std::to_string(out) + ", dev::mx::sde_weight(acc, ex)); }\n"
-               : "                  dev::st(f, " + std::to_string(out) + ", P / den); }\n";
+               : "                  dev::st(f, " + std::to_string(out) + ", dev::fast::div(P, den)); }\n";
     return s;
 }
 
@@ -182,6 +213,7 @@ std::string channel_body(const Compiled& C, size_t c, bool mixed) {
     s += "                dev::load_inputs<kMix>(f, lp, " + cs + ", " + std::to_string(C.n_random) + ", ev, local, active);\n";
     size_t pc = 0;
     InvariantMemo memo;
+    RangeMemo range;
     while (pc < C.code.size() && C.code[pc] != kOpOutput) {
         const int op = C.code[pc], na = C.code[pc + 1], no = C.code[pc + 2];
         const int32_t* a = C.code.data() + pc + 3;
@@ -189,11 +221,44 @@ std::string channel_body(const Compiled& C, size_t c, bool mixed) {
             std::string decl;
             const std::string body = channel_weight_source(C, a, na, mixed, &memo, &decl);
             s += decl + body;
-            for (int i = 0; i < no; ++i) memo.written(a[na + i]);
+            for (int i = 0; i < no; ++i) {
+                memo.written(a[na + i]);
+                range.written(a[na + i], 1);
+            }
             pc += 3 + na + no;
             continue;
         }
-        for (int i = 0; i < no; ++i) memo.written(a[na + i]);
+        // FP64: a 2->2 block reads the t range that its |t| map was bounded by, evaluated once
+        if (!mixed && op == PS_OP_T_INV_MIN_MAX) {
+            const std::string var = "tr" + std::to_string(range.next++);
+            const std::array<int32_t, 5> key = {a[0], a[1], a[2], a[3], a[4]};
+            s += "                dev::TRange " + var + "; { constexpr int32_t a[] = {" + ints(a, na) +
+                 "}; constexpr int32_t o[] = {" + ints(a + na, no) + "}; " + var + " = dev::exec_t_range(a, o, f); }\n";
+            for (int i = 0; i < no; ++i) {
+                memo.written(a[na + i]);
+                range.written(a[na + i], 1);
+            }
+            if (!range.reads(key, a[na], 1) && !range.reads(key, a[na + 1], 1)) range.names[key] = var;
+            pc += 3 + na + no;
+            continue;
+        }
+        if (!mixed && op == PS_OP_TWO_TO_TWO_COM) {
+            const auto it = range.names.find({a[6], a[7], a[8], a[4], a[5]});
+            if (it != range.names.end()) {
+                s += "                { constexpr int32_t a[] = {" + ints(a, na) + "}; constexpr int32_t o[] = {" +
+                     ints(a + na, no) + "}; dev::exec_two_to_two(a, o, f, s_grid, " + it->second + "); }\n";
+                for (int i = 0; i < no; ++i) {
+                    memo.written(a[na + i]);
+                    range.written(a[na + i], out_width(op, i));
+                }
+                pc += 3 + na + no;
+                continue;
+            }
+        }
+        for (int i = 0; i < no; ++i) {
+            memo.written(a[na + i]);
+            range.written(a[na + i], out_width(op, i));
+        }
         s += "                {";
         s += na ? " constexpr int32_t a[] = {" + ints(a, na) + "};" : " const int32_t* a = nullptr;";
         s += no ? " constexpr int32_t o[] = {" + ints(a + na, no) + "};" : " const int32_t* o = nullptr;";
@@ -332,9 +397,9 @@ void dump_source(const std::string& src) {
 std::mutex g_unit_mu;
 std::map<std::string, std::vector<char>> g_units;  // channel unit source -> relocatable cubin
 
-bool split_program(size_t n_ch) {
+bool split_program(size_t n_ch, bool mixed) {
     if (const char* e = std::getenv("PS_JIT_SPLIT")) return e[0] == '1';  // diagnostic override
-    return n_ch > static_cast<size_t>(kJitInlineChannels);
+    return n_ch > static_cast<size_t>(mixed ? kJitInlineMixed : kJitInlineChannels);
 }
 
 // nvJitLink: relocatable cubins -> one executable cubin for sm_103a (host only).
@@ -392,9 +457,16 @@ int register_cap(int block, int min_blocks) {
 
 Plan make_plan(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed) {
     Plan p;
-    p.split = split_program(ch.size());
+    p.split = split_program(ch.size(), mixed);
     if (p.split) {
         p.max_regs = register_cap(block, min_blocks);
+        // Without a request, an FP64 channel whose slot file (two registers a slot) leaves room for the
+        // arithmetic in 168 registers is held to them: 12 warps an SM instead of 8 hide the FP64 latency
+        // (2->5, 60 slots, 4e6 events: 6.5 against 6.9 ms); a larger one would spill (2->8, 85 slots: 5.20
+        // against 4.91 ms per 2^20).
+        int slots = 0;
+        for (const Compiled& c : ch) slots = std::max(slots, c.n_slots);
+        if (!mixed && min_blocks <= 0 && slots <= 60) p.max_regs = register_cap(128, 3);
         p.units = jit_sources_split(ch, block, min_blocks, mixed);
         for (const std::string& u : p.units) p.key += u + "\n// ---- unit\n";
         p.key += "// maxrregcount " + std::to_string(p.max_regs) + "\n";

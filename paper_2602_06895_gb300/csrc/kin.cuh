@@ -3,6 +3,9 @@
 // a 2->2 block.
 #pragma once
 #include <cmath>
+#include <cstdint>
+
+#include "fp64_fast.cuh"
 
 namespace ps {
 namespace dev {
@@ -16,6 +19,10 @@ constexpr long long kInfBits = 0x7FF0000000000000LL;
 __device__ __forceinline__ long long dbits(double v) { return __double_as_longlong(v); }
 // isfinite(v)
 __device__ __forceinline__ bool finite_bits(double v) { return (dbits(v) & kInfBits) != kInfBits; }
+// The same, and v = +-0, on the words: the compiler recognises a test of the 64-bit pattern as a floating-point
+// class test or a comparison, which the FP64 pipe executes (25 and more per event).
+__device__ __forceinline__ bool is_finite(double v) { return (__double2hiint(v) & 0x7FF00000) != 0x7FF00000; }
+__device__ __forceinline__ bool is_zero(double v) { return ((__double2hiint(v) << 1) | __double2loint(v)) == 0; }
 // 0 < v <= 1 (false for NaN)
 __device__ __forceinline__ bool in_unit_bits(double v) {
     const long long b = dbits(v);
@@ -60,6 +67,23 @@ __device__ __forceinline__ double small_to_double(int k) {
     const int msb = 31 - __clz(k);
     const unsigned long long m = (static_cast<unsigned long long>(k) << (52 - msb)) & 0xFFFFFFFFFFFFFULL;
     return __longlong_as_double(static_cast<long long>((static_cast<unsigned long long>(1023 + msb) << 52) | m));
+}
+// y - k for 0 <= k <= floor(y) < 2^31, y >= 0, exactly, from the bits: the fraction below the binary point where k is
+// the floor; another k (a clamped bin) is subtracted as a double
+__device__ __forceinline__ double sub_small(double y, int k) {
+    const uint32_t hi = static_cast<uint32_t>(__double2hiint(y)), lo = static_cast<uint32_t>(__double2loint(y));
+    const int e = static_cast<int>(hi >> 20) - 1023;  // negative y, NaN: out of the range below
+    if (k == 0) return y;
+    const unsigned long long m = ((static_cast<unsigned long long>((hi & 0xFFFFFu) | 0x100000u) << 32) | lo) << 11;
+    const int es = e & 31;
+    const unsigned long long f = m << (es + 1);  // the fraction, in units of 2^-64
+    const int lz = __clzll(static_cast<long long>(f));
+    double v = f == 0 ? 0.0
+                      : __longlong_as_double(static_cast<long long>(((f << (lz & 63)) >> 11) +
+                                                                          (static_cast<unsigned long long>(1021 - lz) << 52)));
+    const bool ok = e >= 0 && e < 31 && static_cast<int>(static_cast<uint32_t>(m >> 32) >> (31 - es)) == k;
+    if (__builtin_expect(!ok, 0)) v = fast::slow_sub(y, small_to_double(k));
+    return v;
 }
 // fmax(a, b) on the bit patterns: doubles order like the integers b ^ (0x7FF..F if negative);
 // a NaN operand gives the other one
@@ -124,6 +148,23 @@ __device__ __forceinline__ double kallen_m(double x, double m1, double m2) {
     }
     return pos_bits(l) ? l : 0.0;
 }
+// kallen_m for the forward kernels (masses compared with zero on their words), and its root: x itself for
+// two massless legs
+__device__ __forceinline__ double kallen_out(double x, double m1, double m2) {
+    double l;
+    if (is_zero(m1) && is_zero(m2)) {
+        l = __dmul_rn(x, x);
+    } else {
+        const double hi = __dadd_rn(m1, m2), lo = __dadd_rn(m1, -m2);
+        l = __dmul_rn(fma(-hi, hi, x), fma(-lo, lo, x));
+    }
+    return pos_bits(l) ? l : 0.0;
+}
+__device__ __forceinline__ double sqrt_kallen_out(double x, double m1, double m2) {
+    if (is_zero(m1) && is_zero(m2)) return x;
+    const double l = kallen_out(x, m1, m2);
+    return pos_bits(l) ? fast::sqrt(l) : 0.0;
+}
 
 // Pure boosts out of the rest frame of q (mass mq) sharing their reciprocals: 1/mq and
 // 1/(mq (E_q + mq)) are taken once per frame, for every momentum boosted with it.
@@ -132,7 +173,7 @@ struct BoostFrame {
     double inv_m, k;    // 1/mq, 1/(mq (E_q + mq))
 };
 __device__ __forceinline__ BoostFrame boost_frame(const P4& q, double mq, double inv_m) {
-    return {q.e, q.x, q.y, q.z, inv_m, 1.0 / (mq * (q.e + mq))};
+    return {q.e, q.x, q.y, q.z, inv_m, fast::rcp(mq * (q.e + mq))};
 }
 __device__ __forceinline__ P4 boost_out(const P4& p, const BoostFrame& b) {
     double qp = b.x * p.x + b.y * p.y + b.z * p.z;
@@ -181,11 +222,64 @@ __device__ __forceinline__ void t_range(double s, double mA2, double mB2, double
     double prod = (m12 - mA2) * (m22 - mB2) + (m12 * mB2 - m22 * mA2) * (m12 - m22 - mA2 + mB2) / s;
     const bool a_nonpos = nonpos_bits(A);       // A <= 0, on the bits
     double big = a_nonpos ? A - B : A + B;      // root without cancellation
-    double small = !zero_bits(big) ? prod / big : 0.0;
+    double small = !is_zero(big) ? prod / big : 0.0;
     double tplus = a_nonpos ? small : big;      // closest to zero
     double tminus = a_nonpos ? big : small;
     tabs_min = -tplus;
     tabs_max = -tminus;
+}
+// Sums and products with a term that may be the constant zero of a compiled channel (massless legs):
+// x + 0 and x * 0 do not fold under IEEE rules, a select on the bits of a constant does.
+__device__ __forceinline__ double add_z(double a, double b) { return is_zero(b) ? a : (is_zero(a) ? b : __dadd_rn(a, b)); }
+__device__ __forceinline__ double sub_z(double a, double b) { return is_zero(b) ? a : (is_zero(a) ? -b : __dadd_rn(a, -b)); }
+__device__ __forceinline__ double mul_z(double a, double b) { return is_zero(a) || is_zero(b) ? 0.0 : __dmul_rn(a, b); }
+
+// kallen(x, y, z) of the incoming legs of a 2->2 block with every rounding spelled out
+__device__ __forceinline__ double kallen_in(double x, double y, double z) {
+    double l;
+    if (is_zero(y) && is_zero(z)) {
+        l = __dmul_rn(x, x);
+    } else if (nonneg_bits(y) && nonneg_bits(z)) {
+        const double ry = fast::sqrt(y), rz = fast::sqrt(z);
+        const double hi = __dadd_rn(ry, rz), lo = __dadd_rn(ry, -rz);
+        l = __dmul_rn(fma(-hi, hi, x), fma(-lo, lo, x));
+    } else if (nonpos_bits(y) && nonpos_bits(z)) {
+        const double d = sub_z(z, y), t = add_z(y, z);  // (x - t)^2 - 4 y z = x (x - 2 t) + d^2, t <= 0
+        l = fma(d, d, __dmul_rn(x, fma(-2.0, t, x)));
+    } else {
+        const double d = __dadd_rn(__dadd_rn(x, -y), -z);
+        l = fma(d, d, __dmul_rn(__dmul_rn(-4.0, y), z));
+    }
+    return pos_bits(l) ? l : 0.0;
+}
+
+// The t range for the forward kernels, with what the block itself needs of it: the Kallen functions of
+// the incoming and outgoing legs and B.  Every rounding is spelled out (no contraction is left to the
+// compiler): the |t| map and the block evaluate it separately, and the distance |t| - |t|_min must be
+// taken from the very bound that |t| was built on.
+struct TRange {
+    double lo, hi, B, lam_in, lam_out;  // |t|_min, |t|_max
+    double e1, e2;                      // s + m1^2 - m2^2, s - m1^2 + m2^2
+};
+__device__ __forceinline__ TRange t_range_fast(double s, double mA2, double mB2, double m1, double m2) {
+    TRange r;
+    const double m12 = __dmul_rn(m1, m1), m22 = __dmul_rn(m2, m2);
+    const double inv_s = fast::rcp(s), inv2s = fast::half(inv_s);
+    r.e1 = sub_z(add_z(s, m12), m22);
+    r.e2 = sub_z(add_z(s, m22), m12);
+    const double A = fma(-__dmul_rn(sub_z(add_z(s, mA2), mB2), r.e1), inv2s, add_z(mA2, m12));
+    r.lam_in = kallen_in(s, mA2, mB2);
+    r.lam_out = kallen_out(s, m1, m2);
+    const double l = __dmul_rn(r.lam_in, r.lam_out);
+    r.B = pos_bits(l) ? __dmul_rn(fast::sqrt(l), inv2s) : 0.0;
+    const double cross = mul_z(sub_z(mul_z(m12, mB2), mul_z(m22, mA2)), add_z(sub_z(sub_z(m12, m22), mA2), mB2));
+    const double prod = fma(cross, inv_s, mul_z(sub_z(m12, mA2), sub_z(m22, mB2)));
+    const bool a_nonpos = nonpos_bits(A);
+    const double big = __dadd_rn(A, a_nonpos ? -r.B : r.B);
+    const double small = is_zero(big) ? 0.0 : fast::div(prod, big);
+    r.lo = -(a_nonpos ? small : big);
+    r.hi = -(a_nonpos ? big : small);
+    return r;
 }
 
 }  // namespace dev

@@ -17,33 +17,32 @@ using rng::philox4x32_10;
 using rng::unit_from_bits;
 
 // ---------------------------------------------------------------- azimuths
-// cos and sin of 2 pi k / kTrigN into t[2k], t[2k+1], from sincospi (once per CTA)
+// cos and sin of 2 pi k / kTrigN into t[2k], t[2k+1], from the table (once per CTA)
 __device__ __forceinline__ void stage_trig(double* t, int tid, int nthreads) {
-    for (int k = tid; k < kTrigN; k += nthreads) {
-        double s, c;
-        sincospi(2.0 * k / kTrigN, &s, &c);
-        t[2 * k] = c;
-        t[2 * k + 1] = s;
-    }
+    for (int k = tid; k < kTrigDoubles; k += nthreads) t[k] = __ldg(&kTrigTab[k]);
 }
 
-// sin and cos of phi = 2 pi r for r in [0, 1], table-driven: r kTrigN = k + f (exact; f in [0, 1)),
-// x = f 2 pi / kTrigN < 0.0246, then sin x and cos x by their Taylor series to x^7 and x^6 (the
-// first omitted terms are below 1e-17 of the result) and the angle-sum formulas with the
-// tabulated point k.  About 15 FP64 operations where sincospi takes about 25; a few ulps.  Other r
-// (outside [0, 1], NaN) take sincospi.
+// sin and cos of phi = 2 pi r for r in [0, 1], table-driven: k the integer nearest r kTrigN (found in
+// FP32), f = r - k / kTrigN (exact), then sin 2 pi f and cos 2 pi f (|2 pi f| < 0.0123) by their Taylor
+// series in f, to f^7 and f^6, the innermost coefficient of each in FP32 (its rounding enters below 2^-55),
+// and the angle-sum formulas with the tabulated point k.  11 FP64 operations where sincospi takes
+// about 25; a few ulps.  Other r (outside [0, 1], NaN) take sincospi.
 __device__ __forceinline__ void sincos_turn(double r, const double* trig, double& s, double& c) {
     if (static_cast<unsigned long long>(dbits(r)) > 0x3FF0000000000000ULL) {  // not in [+0, 1]
         sincospi(2.0 * r, &s, &c);
         return;
     }
-    const double t = r * kTrigN;
-    const int k = floor_small(t);
-    const double f = t - small_to_double(k);
-    const double x = f * (kPi / (kTrigN / 2)), x2 = x * x;
-    const double sx = fma(x * x2, fma(x2, fma(x2, -1.0 / 5040.0, 1.0 / 120.0), -1.0 / 6.0), x);
-    const double cx = fma(x2, fma(x2, fma(x2, -1.0 / 720.0, 1.0 / 24.0), -0.5), 1.0);
-    const int j = 2 * (k & (kTrigN - 1));  // r = 1 is the point k = 0 of the next turn
+    constexpr double t2 = 4.0 * kPi * kPi;  // (2 pi)^2
+    const float kf = rintf(fast::narrow(r) * static_cast<float>(kTrigN));
+    const double f = fma(fast::widen_int(kf), -1.0 / kTrigN, r);
+    const double f2 = f * f;
+    const float g = fast::narrow(f2);
+    const double sp = fast::widen(fmaf(g, static_cast<float>(-2.0 * kPi * t2 * t2 * t2 / 5040.0),
+                                       static_cast<float>(2.0 * kPi * t2 * t2 / 120.0)));
+    const double cp = fast::widen(fmaf(g, static_cast<float>(-t2 * t2 * t2 / 720.0), static_cast<float>(t2 * t2 / 24.0)));
+    const double sx = f * fma(f2, fma(f2, sp, -2.0 * kPi * t2 / 6.0), 2.0 * kPi);
+    const double cx = fma(f2, fma(f2, cp, -0.5 * t2), 1.0);
+    const int j = 2 * (static_cast<int>(kf) & (kTrigN - 1));  // k = kTrigN is the point 0 of the next turn
     const double ck = trig[j], sk = trig[j + 1];
     s = fma(sk, cx, ck * sx);
     c = fma(ck, cx, -(sk * sx));
@@ -55,21 +54,23 @@ __device__ __forceinline__ void sincos_turn(double r, const double* trig, double
 // 1e-19 of it), and the addition theorem as a correction of the tabulated point,
 //   tan(k h + y) = tan(k h) + tan y (1 + tan^2 k h) / (1 - tan(k h) tan y),
 // with tan(k h) a double-double and a non-negative correction (no cancellation).  Within 1.5 ulps,
-// and the correctly rounded value for about 99 % of arguments (an emulation on the host against
-// 80-bit tanl), in about 17 FP64 operations where tan takes about 29.  k is clamped to the table,
+// and the correctly rounded value for about 99 % of arguments, in 13 FP64 operations where tan takes
+// about 29.  k is clamped to the table,
 // so every argument reads inside it; beyond pi/4 the value is not the tangent (map_bw never
 // passes one).
 __device__ __forceinline__ double tan_quarter(double x) {
     const long long sign = dbits(x) & static_cast<long long>(0x8000000000000000ULL);
     const double ax = __longlong_as_double(dbits(x) ^ sign);
-    const int k = min(floor_small(ax * kTanInvH), kTanN);
-    const double kd = small_to_double(k);
+    // k from FP32: at a boundary it may be one off, and y a rounding outside [0, h)
+    const int k = max(min(static_cast<int>(fast::narrow(ax) * static_cast<float>(kTanInvH)), kTanN), 0);
+    const double kd = fast::widen_int(static_cast<float>(k));
     const double y = fma(-kd, kTanH2, fma(-kd, kTanH1, ax));
     const double y2 = y * y;
-    const double p = fma(y2, fma(y2, 17.0 / 315.0, 2.0 / 15.0), 1.0 / 3.0);
+    const double p =  // the inner terms, below 2^-29 of tan y, in FP32
+        fma(y2, fast::widen(fmaf(fast::narrow(y2), 17.0f / 315.0f, 2.0f / 15.0f)), 1.0 / 3.0);
     const double ty = fma(y * y2, p, y);
     const double th = __ldg(&kTanHi[k]);
-    const double c = (ty * __ldg(&kTanSq1[k])) / fma(-th, ty, 1.0);
+    const double c = fast::div(ty * __ldg(&kTanSq1[k]), fma(-th, ty, 1.0));
     const double t = th + (__ldg(&kTanLo[k]) + c);
     return __longlong_as_double(dbits(t) | sign);
 }
@@ -81,32 +82,91 @@ __device__ __forceinline__ double tan_quarter(double x) {
 //   nu == 1: x = x_min + lo expm1(r L),              J = (x - m^2) L
 //   nu <  1: z = r expm1(w L),  x = x_min + lo expm1(log1p(z)/w),  J = (x - m^2) rho/(w (1+z))
 //   nu >  1: z = (1-r) expm1(-w L), x - m^2 = hi exp(log1p(z)/w), J = -(x - m^2) rho'/(w (1+z))
-__device__ __forceinline__ bool map_nu(double r, double m, double nu, double xmin, double xmax, double a,
-                                       double& x, double& jac) {
-    double m2 = pos_bits(m) ? m * m : -a;
-    double lo = xmin - m2, hi = xmax - m2;
-    bool ok = pos_bits(lo) && ge_pos_bits(hi, lo);
-    double L = log1p((xmax - xmin) / lo);
+//
+// When 1/w is an integer n = 2..6 up to rounding (nu = 0.8, the default, and 0.5, 2/3, 3/4 ...) the power and
+// the root of nu < 1 are taken without logarithms: rho = (1 + p)^w - 1 solves rho S_n(1 + rho) = p and
+// (1 + z)^(1/w) - 1 = z S_n(1 + z), S_n(u) = 1 + u + ... + u^(n-1).  The double w is n w = 1 - eta, eta of a
+// few 1e-16: its first order, (1 + p)^-eta and (1 + z)^(n eta), is kept, so that the map is that of
+// the given nu.  About 30 FP64 instructions where the logarithms and exponentials take about 65 (and
+// CUDA's took 140); a channel of pure t-chain makes seven such maps.
+// have_L: L comes in as a constant of the channel (both bounds are immediates).
+struct NuOut {
+    double x, jac;
+};
+// Any exponent, by logarithms and exponentials; p = (x_max - x_min)/lo.
+__device__ __forceinline__ NuOut map_nu_general(double r, double nu, double xmin, double lo, double hi, double m2, double p,
+                                                bool have_L, double L_in) {
+    NuOut o;
+    const double L = have_L ? L_in : fast::log1p(p);
+    const double w = __dadd_rn(1.0, -nu);
     if (dbits(nu) == dbits(1.0)) {
-        double e = expm1(r * L);
-        double xm = fma(lo, e, lo);
-        x = fma(lo, e, xmin);
-        jac = xm * L;
+        const double e = fast::expm1(__dmul_rn(r, L));
+        o.x = fma(lo, e, xmin);
+        o.jac = __dmul_rn(fma(lo, e, lo), L);
     } else if (dbits(nu) < dbits(1.0)) {  // nu < 1 (nu is never NaN)
-        double w = 1.0 - nu;
-        double rho = expm1(w * L);
-        double z = r * rho;
-        double e = expm1(log1p(z) / w);
-        double xm = fma(lo, e, lo);
-        x = fma(lo, e, xmin);
-        jac = xm * rho / (w * (1.0 + z));
+        const double rho = fast::expm1(__dmul_rn(w, L));
+        const double z = __dmul_rn(r, rho);
+        const double e = fast::expm1(fast::div(fast::log1p(z), w));
+        o.x = fma(lo, e, xmin);
+        o.jac = fast::div(__dmul_rn(fma(lo, e, lo), rho), __dmul_rn(w, __dadd_rn(1.0, z)));
     } else {
-        double w = 1.0 - nu;
-        double rho = expm1(-w * L);
-        double z = (1.0 - r) * rho;
-        double xm = hi * exp(log1p(z) / w);
-        x = m2 + xm;
-        jac = -xm * rho / (w * (1.0 + z));
+        const double rho = fast::expm1(__dmul_rn(-w, L));
+        const double z = __dmul_rn(__dadd_rn(1.0, -r), rho);
+        const double xm = __dmul_rn(hi, fast::exp(fast::div(fast::log1p(z), w)));
+        o.x = __dadd_rn(m2, xm);
+        o.jac = fast::div(__dmul_rn(-xm, rho), __dmul_rn(w, __dadd_rn(1.0, z)));
+    }
+    return o;
+}
+static __device__ __noinline__ NuOut map_nu_far(double r, double nu, double xmin, double lo, double hi, double m2, double p) {
+    return map_nu_general(r, nu, xmin, lo, hi, m2, p, false, 0.0);
+}
+
+// const_nu: nu is a constant of a compiled channel, and the choice of the form folds; ranges beyond the
+// root's (p outside [2^-60, 2^100)) then take one out-of-line copy of the general form.
+__device__ __forceinline__ bool map_nu(double r, double m, double nu, double xmin, double xmax, double a,
+                                       double& x, double& jac, bool have_L, double L_in, bool const_nu) {
+    double m2 = pos_bits(m) ? __dmul_rn(m, m) : -a;
+    const double lo = __dadd_rn(xmin, -m2), hi = __dadd_rn(xmax, -m2);
+    bool ok = pos_bits(lo) && ge_pos_bits(hi, lo);
+    const double range = sub_z(xmax, xmin);
+    const double p = have_L && const_nu ? range / lo : fast::div(range, lo);
+    const double w = __dadd_rn(1.0, -nu);
+    const float wf = const_nu ? static_cast<float>(w) : fast::narrow(w);
+    const float nf = rintf(const_nu ? 1.0f / wf : fast::rcp_approx(wf));
+    const bool near = wf > 0.15f && wf < 0.55f && fabsf(fmaf(-nf, wf, 1.0f)) < 1e-6f;
+    const double nd = const_nu ? static_cast<double>(nf) : fast::widen(near ? nf : 1.0f);
+    const double eta = fma(-nd, w, 1.0);
+    const float ef = const_nu ? static_cast<float>(eta) : fast::narrow(eta);
+    const bool whole = near && fabsf(ef) < 1e-13f;
+    const bool in_range = fast::hi32(p) - 0x3C300000u < 0x0A000000u;
+    if (whole && (const_nu || in_range)) {
+        const int n = static_cast<int>(nf);
+        const float pf = fast::narrow(p);
+        // 1 + p to the power -eta: p' = p - eta (1 + p) log(1 + p)
+        const float dp = ef * (1.0f + pf) * (0.693147181f * fast::lg2_approx(1.0f + pf));
+        const double rho = fast::root1p(ef != 0.0f ? __dadd_rn(p, -fast::widen_or_zero(dp)) : p, n);
+        const double z = __dmul_rn(r, rho), u = __dadd_rn(1.0, z);
+        double s_prev, s_n;
+        fast::geometric(u, n, s_prev, s_n);
+        double e = __dmul_rn(z, s_n), pw = fma(z, s_prev, 1.0);  // u^n - 1 and u^(n-1)
+        if (ef != 0.0f) {
+            const float uf = fast::narrow(u), pwf = fast::narrow(pw);
+            const float d = pwf * (nf * ef) * (0.693147181f * fast::lg2_approx(uf));
+            e = __dadd_rn(e, fast::widen_or_zero(d * uf));
+            pw = __dadd_rn(pw, fast::widen_or_zero(d));
+        }
+        x = fma(lo, e, xmin);
+        jac = __dmul_rn(__dmul_rn(__dmul_rn(lo, rho), pw), fma(nd, eta, nd));  // 1/w = n (1 + eta)
+        if (const_nu && __builtin_expect(!in_range, 0)) {
+            const NuOut o = map_nu_far(r, nu, xmin, lo, hi, m2, p);
+            x = o.x;
+            jac = o.jac;
+        }
+    } else {
+        const NuOut o = map_nu_general(r, nu, xmin, lo, hi, m2, p, have_L, L_in);
+        x = o.x;
+        jac = o.jac;
     }
     x = clamp_nonneg(x, xmin, xmax);  // the map lands in [x_min, x_max] (rounding at the ends)
     if (!ok) { x = xmin; jac = 0.0; }
@@ -125,22 +185,24 @@ __device__ __forceinline__ bool map_nu(double r, double m, double nu, double xmi
 // its own formula.  u1 = atan(a) may come in as the channel's constant (x_min immediate);
 // have_u1 selects it.
 __device__ __forceinline__ bool map_bw(double r, double M, double G, double xmin, double xmax,
-                                       double& x, double& jac, bool have_u1 = false, double u1 = 0.0) {
-    double mg = M * G, m2 = M * M;
+                                       double& x, double& jac, bool have_u1, double u1, bool const_width) {
+    // every rounding is spelled out: a compiled channel could contract differently where constants fold and
+    // where a bound is the product of the op before
+    const double mg = __dmul_rn(M, G), m2 = __dmul_rn(M, M);
     bool ok = pos_bits(mg) && ge_pos_bits(xmax, xmin);  // x_min >= 0 here (a squared mass)
-    double inv_mg = 1.0 / mg;
-    double a = (xmin - m2) * inv_mg, b = (xmax - m2) * inv_mg;
-    double D = atan2((xmax - xmin) * inv_mg, fma(a, b, 1.0));
-    double u = (have_u1 ? u1 : atan(a)) + D * r;
+    double inv_mg = const_width ? 1.0 / mg : fast::rcp(mg);  // a constant of a compiled channel folds
+    const double a = __dmul_rn(__dadd_rn(xmin, -m2), inv_mg), b = __dmul_rn(__dadd_rn(xmax, -m2), inv_mg);
+    const double D = fast::atan2(__dmul_rn(sub_z(xmax, xmin), inv_mg), fma(a, b, 1.0));
+    const double Dr = __dmul_rn(D, r), u = __dadd_rn(have_u1 ? u1 : fast::atan(a), Dr);
     bool low = below_neg_bits(u, 0.25 * kPi), high = above_pos_bits(u, 0.25 * kPi);
-    double arg = low ? D * r : (high ? D * (1.0 - r) : u);
-    double T = tan_quarter(arg);
-    const double den = low ? 1.0 - a * T : (high ? 1.0 + b * T : 1.0);
-    const double num = low ? T * (1.0 + a * a) : (high ? b - T : T);
-    const double kk = low ? 1.0 + a * a : (high ? 1.0 + b * b : 1.0);
-    const double rd = 1.0 / den;
-    x = (low ? xmin : m2) + mg * (num * rd);
-    jac = D * mg * (kk * (1.0 + T * T) * (rd * rd));
+    const double T = tan_quarter(low ? Dr : (high ? __dmul_rn(D, __dadd_rn(1.0, -r)) : u));
+    const double a2 = fma(a, a, 1.0), b2 = fma(b, b, 1.0);
+    const double den = low ? fma(-a, T, 1.0) : (high ? fma(b, T, 1.0) : 1.0);
+    const double num = low ? __dmul_rn(T, a2) : (high ? __dadd_rn(b, -T) : T);
+    const double kk = low ? a2 : (high ? b2 : 1.0);
+    const double rd = fast::rcp(den);
+    x = fma(mg, __dmul_rn(num, rd), low ? xmin : m2);
+    jac = __dmul_rn(__dmul_rn(D, mg), __dmul_rn(__dmul_rn(kk, fma(T, T, 1.0)), __dmul_rn(rd, rd)));
     x = clamp_nonneg(x, xmin, xmax);
     if (!ok) { x = xmin; jac = 0.0; }
     return ok;
@@ -150,49 +212,42 @@ __device__ __forceinline__ bool map_bw(double r, double M, double G, double xmin
 // frame of p0 = pA + pB; cos(theta) from |t| via 1 -+ cos = (|t| - |t|_min)/B resp.
 // (|t|_max - |t|)/B, whichever is smaller; the momentum is rotated by R(phi_A, theta_A)
 // = Rz(phi_A) Ry(theta_A) (Sec. 2.2.6) and boosted back.
-__device__ __forceinline__ double two_to_two(double rphi, P4 pA, P4 pB, double tabs, double m1, double m2,
-                                             double s, double mA2, double mB2, P4& p1, P4& p2,
-                                             const double* trig) {
+__device__ __forceinline__ double two_to_two(double rphi, P4 pA, P4 pB, double tabs, double s, const TRange& tr,
+                                             P4& p1, P4& p2, const double* trig) {
     P4 p0 = p4_add(pA, pB);
-    double m0 = sqrt(s);
-    // 1/m0 = m0/s and the boost's 1/(m0 (E0 + m0)) from one division, R = 1/(s (E0 + m0))
-    const double ep = p0.e + m0;
-    const double R = 1.0 / (s * ep);
-    const BoostFrame bf{p0.e, p0.x, p0.y, p0.z, m0 * (ep * R), m0 * R};
+    double inv_m0;
+    double m0 = fast::sqrt_rcp(s, inv_m0);
+    const BoostFrame bf{p0.e, p0.x, p0.y, p0.z, inv_m0, fast::rcp(m0 * (p0.e + m0))};
     P4 a = boost_in(pA, bf);
     double pt2 = a.x * a.x + a.y * a.y;
     bool has_pt = pos_bits(pt2);
-    double ipt = has_pt ? rsqrt(pt2) : 0.0;
+    double ipt = has_pt ? fast::rsqrt(pt2) : 0.0;
     double pt = pt2 * ipt;
-    double rp = rsqrt(pt2 + a.z * a.z);
+    double rp = fast::rsqrt(pt2 + a.z * a.z);
     double ca = a.z * rp, sa = pt * rp;
     double cpa = has_pt ? a.x * ipt : 1.0, spa = has_pt ? a.y * ipt : 0.0;
 
-    double tlo, thi, B;
-    t_range(s, mA2, mB2, m1, m2, tlo, thi, B);
-    double dlo = tabs - tlo, dhi = thi - tabs;
+    double dlo = tabs - tr.lo, dhi = tr.hi - tabs;
     bool near_lo = dlo <= dhi;
-    const bool b_pos = pos_bits(B);  // B > 0, on the bits
-    double iB = b_pos ? 1.0 / B : 0.0;
-    double first = (near_lo ? dlo : dhi) * iB;  // 1 - cos (near_lo) or 1 + cos
+    const bool b_pos = pos_bits(tr.B);  // B > 0, on the bits
+    double first = b_pos ? fast::div(near_lo ? dlo : dhi, tr.B) : 0.0;  // 1 - cos (near_lo) or 1 + cos
     double omc = b_pos ? (near_lo ? first : 2.0 - first) : 1.0;
     double opc = b_pos ? (near_lo ? 2.0 - first : first) : 1.0;
     double cth = (omc <= opc) ? 1.0 - omc : opc - 1.0;
     const double so = omc * opc;
-    double sth = sqrt(pos_bits(so) ? so : 0.0);
+    double sth = pos_bits(so) ? fast::sqrt(so) : 0.0;
     double sph, cph;
     sincos_turn(rphi, trig, sph, cph);
 
-    double m12 = m1 * m1, m22 = m2 * m2;
-    double i2m0 = 0.5 * bf.inv_m;
-    double pabs = sqrt(kallen_m(s, m1, m2)) * i2m0;
-    double e1 = (s + m12 - m22) * i2m0, e2 = (s + m22 - m12) * i2m0;
+    double i2m0 = fast::half(bf.inv_m);
+    double pabs = (pos_bits(tr.lam_out) ? fast::sqrt(tr.lam_out) : 0.0) * i2m0;
+    double e1 = tr.e1 * i2m0, e2 = tr.e2 * i2m0;
     double vx = pabs * sth * cph, vy = pabs * sth * sph, vz = pabs * cth;
     // Ry(theta_A) then Rz(phi_A)
     double rx = ca * vx + sa * vz, rz = -sa * vx + ca * vz;
     P4 q1 = {e1, cpa * rx - spa * vy, spa * rx + cpa * vy, rz};
     boost_out_pair(q1, e2, bf, p1, p2);
-    return 0.5 * kPi * rsqrt(kallen(s, mA2, mB2));
+    return 0.5 * kPi * fast::rsqrt(tr.lam_in);
 }
 
 // 1->2 decay in (phi, theta), Sec. 2.2.3: cos = 2 r_theta - 1, sin = 2 sqrt(r_theta (1 - r_theta)),
@@ -200,22 +255,30 @@ __device__ __forceinline__ double two_to_two(double rphi, P4 pA, P4 pB, double t
 template <bool kBoost>
 __device__ __forceinline__ double two_body(double rphi, double rth, double s0, double m1, double m2, P4 p0,
                                            P4& p1, P4& p2, const double* trig) {
-    double m0 = sqrt(s0);
-    // 1/s0 by its own division: the Jacobian sqrt(lambda)/s0 must not pick up the rounding of the
-    // parent's energy (as a reciprocal shared with the boost's 1/(m0 (E0 + m0)) would)
-    const double inv_s0 = 1.0 / s0;
-    const double inv_m0 = m0 * inv_s0;  // 1/m0 = m0/s0
-    double m12 = m1 * m1, m22 = m2 * m2;
-    // sqrt(lambda) = s0 exactly for two massless daughters
-    double sl = (zero_bits(m12) && zero_bits(m22)) ? s0 : sqrt(kallen_m(s0, m1, m2));
-    double i2m0 = 0.5 * inv_m0;
-    double pabs = sl * i2m0;
-    double e1 = (s0 + m12 - m22) * i2m0, e2 = (s0 + m22 - m12) * i2m0;
+    double inv_m0;
+    const double m0 = fast::sqrt_rcp(s0, inv_m0);
+    double pabs, e1, e2, jac;
+    if (is_zero(m1) && is_zero(m2)) {
+        // massless daughters: |p| = E1 = E2 = m0/2 and sqrt(lambda)/s0 = 1 (NaN where s0 is not positive and finite)
+        pabs = e1 = e2 = fast::half(m0);
+        jac = pos_bits(s0) && is_finite(s0) ? 0.5 * kPi : __longlong_as_double(0x7FF8000000000000LL);
+    } else {
+        double m12 = m1 * m1, m22 = m2 * m2;
+        const double sl = sqrt_kallen_out(s0, m1, m2);
+        double i2m0 = fast::half(inv_m0);
+        pabs = sl * i2m0;
+        const double dm = m12 - m22;
+        e1 = (s0 + dm) * i2m0, e2 = (s0 - dm) * i2m0;
+        // its own quotient: the Jacobian must not pick up the rounding of the parent's energy
+        jac = 0.5 * kPi * fast::div(sl, s0);
+    }
     double cth = 2.0 * rth - 1.0;
-    double sth = 2.0 * sqrt(rth * (1.0 - rth));
+    const double sc = rth * (1.0 - rth);
+    double sth = fast::twice(fast::sqrt(sc));
     double sph, cph;
     sincos_turn(rphi, trig, sph, cph);
-    P4 q1 = {e1, pabs * sth * cph, pabs * sth * sph, pabs * cth};
+    const double pt = pabs * sth;
+    P4 q1 = {e1, pt * cph, pt * sph, pabs * cth};
     P4 q2 = {e2, -q1.x, -q1.y, -q1.z};
     if (kBoost) {
         boost_out_pair(q1, e2, boost_frame(p0, m0, inv_m0), p1, p2);
@@ -223,7 +286,7 @@ __device__ __forceinline__ double two_body(double rphi, double rth, double s0, d
         p1 = q1;
         p2 = q2;
     }
-    return 0.5 * kPi * sl * inv_s0;
+    return jac;
 }
 
 // ---------------------------------------------------------------- interpreter
@@ -318,7 +381,7 @@ __device__ __forceinline__ void sde_factor_s(double& den, double& P, double s, i
     const double d = s - M * M, mg = M * G;
     den *= (kind == 1) ? d * d : fma(d, d, mg * mg);
     if (above_pos_bits(den, 1e200)) {  // keep the running product in range
-        P /= den;
+        P = fast::slow_div(P, den);
         den = 1.0;
     }
 }
@@ -339,6 +402,26 @@ __device__ __forceinline__ void stage_grid(T* s, const double* g, int dims, int 
     }
 }
 
+// The t range of a 2->2 block, and the block from its range (a compiled channel passes the range on, from the
+// op that gave the |t| map its bounds to the block that reads it; the interpreter evaluates it twice).
+template <class Fr>
+__device__ __forceinline__ TRange exec_t_range(const int32_t* a, const int32_t* o, const Fr& f) {
+    const TRange r = t_range_fast(ld(f, a[0]), ld(f, a[1]), ld(f, a[2]), ld(f, a[3]), ld(f, a[4]));
+    st(f, o[0], r.lo);
+    st(f, o[1], r.hi);
+    return r;
+}
+template <class Fr>
+__device__ __forceinline__ void exec_two_to_two(const int32_t* a, const int32_t* o, const Fr& f, const double* grid,
+                                                const TRange& tr) {
+    P4 p1, p2;
+    const double j = two_to_two(ld(f, a[0]), ldp(f, a[1]), ldp(f, a[2]), ld(f, a[3]), ld(f, a[6]), tr, p1, p2,
+                                grid - kTrigDoubles);
+    stp(f, o[0], p1);
+    stp(f, o[1], p2);
+    st(f, o[2], j);
+}
+
 // One instruction of the FP64 interpreter on frame Fr (the shared-memory slot file of the
 // interpreter kernel, or the register frame of a compiled channel).  grid: the channel's staged
 // VEGAS grid in shared memory, preceded by the azimuth table (grid - kTrigDoubles).
@@ -356,13 +439,13 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
                 const bool pow2 = (vbins & (vbins - 1)) == 0 && q * na <= 1000;
                 op_loop<Fr>(0, na, 1, [&](int j) {
                     double r = ld(f, a[j]);
-                    double rn = r * nb;
+                    double rn = pow2 && q < 60 ? fast::mul2(r, q) : r * nb;
                     // the bin and its double from the bits (no FP64-pipe conversions)
                     int k = min(floor_small(rn), vbins - 1);
                     k = max(k, 0);
                     const double e0 = grid[j * (vbins + 1) + k];
                     const double wdt = grid[na * (vbins + 1) + j * vbins + k];  // staged e[k+1] - e[k]
-                    st(f, o[j], fma(rn - small_to_double(k), wdt, e0));
+                    st(f, o[j], fma(sub_small(rn, k), wdt, e0));
                     jac *= pow2 ? wdt : nb * wdt;
                 });
                 if (pow2) jac *= __longlong_as_double(static_cast<long long>(1023 + q * na) << 52);
@@ -371,7 +454,8 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
             }
             case PS_OP_INVARIANT_NU: {
                 double x, j;
-                map_nu(ld(f, a[0]), ld(f, a[1]), ld(f, a[2]), ld(f, a[3]), ld(f, a[4]), ld(f, a[5]), x, j);
+                map_nu(ld(f, a[0]), ld(f, a[1]), ld(f, a[2]), ld(f, a[3]), ld(f, a[4]), ld(f, a[5]), x, j,
+                       na > 6, na > 6 ? ld(f, a[6]) : 0.0, Fr::kStatic);
                 st(f, o[0], x);
                 st(f, o[1], j);
                 break;
@@ -379,7 +463,7 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
             case PS_OP_INVARIANT_BW: {
                 double x, j;
                 map_bw(ld(f, a[0]), ld(f, a[1]), ld(f, a[2]), ld(f, a[3]), ld(f, a[4]), x, j, na > 5,
-                       na > 5 ? ld(f, a[5]) : 0.0);
+                       na > 5 ? ld(f, a[5]) : 0.0, Fr::kStatic);
                 st(f, o[0], x);
                 st(f, o[1], j);
                 break;
@@ -388,13 +472,13 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
                 double r = ld(f, a[0]), shat = ld(f, a[1]), S = ld(f, a[2]);
                 // 1/S once (a constant that a compiled program folds; S is the collider's), then
                 // products in place of the two divisions by S
-                const double iS = 1.0 / S;
+                const double iS = Fr::kStatic ? 1.0 / S : fast::rcp(S);
                 const double tau = shat * iS;
-                double L = log(tau);
-                const double l1 = r * L, l2 = (1.0 - r) * L;  // log x1, log x2
-                const double x1 = exp(l1);
+                double L = fast::log(tau);
+                const double l1 = __dmul_rn(r, L), l2 = __dadd_rn(L, -l1);  // log x1, log x2: their sum is log tau again
+                const double x1 = fast::exp(l1);
                 st(f, o[0], x1);
-                st(f, o[1], tau / x1);  // x1 x2 = tau: a division where a second exponential was
+                st(f, o[1], fast::div(tau, x1));  // x1 x2 = tau: a division where a second exponential was
                 st(f, o[2], -L * iS);
                 if (no > 3) {
                     st(f, o[3], l1);
@@ -403,26 +487,18 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
                 break;
             }
             case PS_OP_COM_P_IN: {
-                double h = 0.5 * ld(f, a[0]);
+                double h = fast::half(ld(f, a[0]));
                 stp(f, o[0], P4{h, 0.0, 0.0, h});
                 stp(f, o[1], P4{h, 0.0, 0.0, -h});
                 break;
             }
             case PS_OP_T_INV_MIN_MAX: {
-                double lo, hi, B;
-                t_range(ld(f, a[0]), ld(f, a[1]), ld(f, a[2]), ld(f, a[3]), ld(f, a[4]), lo, hi, B);
-                st(f, o[0], lo);
-                st(f, o[1], hi);
+                exec_t_range(a, o, f);
                 break;
             }
             case PS_OP_TWO_TO_TWO_COM: {
-                P4 p1, p2;
-                double j = two_to_two(ld(f, a[0]), ldp(f, a[1]), ldp(f, a[2]), ld(f, a[3]), ld(f, a[4]),
-                                      ld(f, a[5]), ld(f, a[6]), ld(f, a[7]), ld(f, a[8]), p1, p2,
-                                      grid - kTrigDoubles);
-                stp(f, o[0], p1);
-                stp(f, o[1], p2);
-                st(f, o[2], j);
+                exec_two_to_two(a, o, f, grid,
+                                t_range_fast(ld(f, a[6]), ld(f, a[7]), ld(f, a[8]), ld(f, a[4]), ld(f, a[5])));
                 break;
             }
             case PS_OP_TWO_BODY_DECAY: {
@@ -447,13 +523,12 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
                 // light-cone form of the longitudinal boost: E+p_z scales by rho = sqrt(x1/x2),
                 // E-p_z by 1/rho (no cancellation for extreme boosts)
                 double x1 = ld(f, a[na - 2]), x2 = ld(f, a[na - 1]);
-                const double t = rsqrt(x1 * x2);  // rho = sqrt(x1/x2) = x1 t, 1/rho = x2 t
-                double rho = x1 * t;
-                double irho = x2 * t;
+                const double t = fast::half(fast::rsqrt(x1 * x2));  // rho = sqrt(x1/x2) = 2 x1 t, 1/rho = 2 x2 t
+                const double hp = x1 * t, hm = x2 * t;              // rho/2, 1/(2 rho)
                 op_loop<Fr>(0, na - 2, 1, [&](int k) {
                     P4 p = ldp(f, a[k]);
-                    double plus = rho * (p.e + p.z), minus = (p.e - p.z) * irho;
-                    stp(f, o[k], P4{0.5 * (plus + minus), p.x, p.y, 0.5 * (plus - minus)});
+                    const double plus = hp * (p.e + p.z), minus = p.e - p.z;
+                    stp(f, o[k], P4{fma(hm, minus, plus), p.x, p.y, fma(-hm, minus, plus)});
                 });
                 break;
             }
@@ -465,10 +540,10 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
             }
             case PS_OP_CUT_UNPHYSICAL: {
                 double w = ld(f, a[0]), x1 = ld(f, a[1]), x2 = ld(f, a[2]);
-                bool bad = !finite_bits(w) || !(in_unit_bits(x1) && in_unit_bits(x2));
+                bool bad = !is_finite(w) || !(in_unit_bits(x1) && in_unit_bits(x2));
                 op_loop<Fr>(3, na, 1, [&](int k) {
                     P4 p = ldp(f, a[k]);
-                    bad |= !(finite_bits(p.e) && finite_bits(p.x) && finite_bits(p.y) && finite_bits(p.z));
+                    bad |= !(is_finite(p.e) && is_finite(p.x) && is_finite(p.y) && is_finite(p.z));
                 });
                 if (bad && active) atomicAdd(cut_count, 1ULL);
                 st(f, o[0], bad ? 0.0 : w);
@@ -477,8 +552,8 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
             case PS_OP_ADD: st(f, o[0], ld(f, a[0]) + ld(f, a[1])); break;
             case PS_OP_SUB: st(f, o[0], ld(f, a[0]) - ld(f, a[1])); break;
             case PS_OP_MUL: st(f, o[0], ld(f, a[0]) * ld(f, a[1])); break;
-            case PS_OP_DIV: st(f, o[0], ld(f, a[0]) / ld(f, a[1])); break;
-            case PS_OP_SQRT: st(f, o[0], sqrt(ld(f, a[0]))); break;
+            case PS_OP_DIV: st(f, o[0], fast::div(ld(f, a[0]), ld(f, a[1]))); break;
+            case PS_OP_SQRT: st(f, o[0], fast::sqrt(ld(f, a[0]))); break;
             case PS_OP_SQUARE: { double v = ld(f, a[0]); st(f, o[0], v * v); break; }
             case PS_OP_MAX: st(f, o[0], fmax_bits(ld(f, a[0]), ld(f, a[1]))); break;
             case PS_OP_MOM_ADD: stp(f, o[0], p4_add(ldp(f, a[0]), ldp(f, a[1]))); break;
@@ -487,11 +562,12 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
                 // one density, or the pair f(x1) f(x2) = exp(alpha (log x1 + log x2)) (1-x1)^b (1-x2)^b
                 const bool pair = na == 6;
                 double x = ld(f, a[0]), al = ld(f, a[1]), be = ld(f, a[2]);
-                double lx = na > 3 ? ld(f, a[3]) : log(x);
+                double lx = na > 3 ? ld(f, a[3]) : fast::log(x);
                 // an add that is never contracted with the product forming log x2 (a compiled
                 // program could fuse them; the interpreter's slot file rounds the product)
                 if (pair) lx = __dadd_rn(lx, ld(f, a[5]));
-                double fx = exp(al * lx);
+                const double v = __dmul_rn(al, lx);  // its rounding, an ulp of log x times alpha, would be the largest error of f
+                double fx = fast::exp(v, fma(al, lx, -v));
                 auto pw = [&](double y) {
                     if (be == 3.0) return y * y * y;
                     if (be == 2.0) return y * y;
@@ -506,13 +582,13 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
             }
             case PS_OP_PROPAGATOR: {
                 double s = ld(f, a[0]), M = ld(f, a[1]), G = ld(f, a[2]);
-                double d = s - M * M;
-                st(f, o[0], 1.0 / (d * d + M * M * G * G));
+                const double d = __dadd_rn(s, -__dmul_rn(M, M)), mg = __dmul_rn(M, G);
+                st(f, o[0], fast::rcp(fma(d, d, __dmul_rn(mg, mg))));
                 break;
             }
             case PS_OP_ONE_PLUS_COS2: {
                 P4 p = ldp(f, a[0]);
-                double c2 = p.z * p.z / (p.x * p.x + p.y * p.y + p.z * p.z);
+                double c2 = fast::div(p.z * p.z, p.x * p.x + p.y * p.y + p.z * p.z);
                 st(f, o[0], 1.0 + c2);
                 break;
             }
@@ -532,7 +608,7 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
                     });
                     sde_factor(den, P, q, kind, M, G);
                 });
-                st(f, o[0], P / den);
+                st(f, o[0], fast::div(P, den));
                 break;
             }
             default: break;

@@ -18,12 +18,13 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
     return c;
 }
 
-// (k + 1/2) 2^-52 for the top 52 bits k of (hi:lo), exactly: the double 1 + k 2^-52 is
-// assembled from bits and (1 - 2^-53) subtracted, which is exact by Sterbenz's lemma.
+// (k + 1/2) 2^-52 for the top 52 bits k of (hi:lo), exactly: the odd integer 2k + 1 < 2^53 in units of
+// 2^-53, its leading bit moved to bit 52 and the exponent set by the integer ALU (no FP64 instruction).
 __device__ __forceinline__ double unit_from_bits(uint32_t hi, uint32_t lo) {
-    unsigned long long k = ((static_cast<unsigned long long>(hi) << 32) | lo) >> 12;
-    double one_plus = __longlong_as_double(0x3FF0000000000000ULL | k);
-    return one_plus - 0x1.fffffffffffffp-1;
+    const unsigned long long m = (((static_cast<unsigned long long>(hi) << 32) | lo) >> 11) | 1ULL;
+    const int lz = __clzll(static_cast<long long>(m));  // 11..63
+    // the leading bit adds one to the exponent field
+    return __longlong_as_double(static_cast<long long>((m << (lz - 11)) + (static_cast<unsigned long long>(1032 - lz) << 52)));
 }
 
 // The float form of a point coordinate, for the mixed-precision programs: (k + 1/2) 2^-23 for the

@@ -105,9 +105,10 @@ void count_launches(int n);
 // (launch bounds; the split form's channel units get the matching register cap).
 std::string jit_source(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed);
 int jit_compile(const std::string& src, std::vector<char>* cubin, std::string* log, bool relocatable, int max_regs);
-// Programs of more than this many channels are compiled one unit per channel, in parallel, and
-// linked: one unit of all channels compiles in time that grows faster than the channel count.
-constexpr int kJitInlineChannels = 6;
+// Programs of more channels than these are compiled one unit per channel, in parallel, and linked: one
+// unit of all channels compiles in time that grows faster than the channel count.  FP64 units are
+// longer (six 2->5 channels: 14.5 s as one unit, 2.3 s as six, the kernel 5% slower), mixed ones shorter.
+constexpr int kJitInlineChannels = 2, kJitInlineMixed = 6;
 std::vector<std::string> jit_sources_split(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed);
 // The program's kernel as one executable cubin: a single unit, or the split units linked.
 int jit_build(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, std::vector<char>* cubin,
