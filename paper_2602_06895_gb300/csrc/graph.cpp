@@ -1730,7 +1730,7 @@ int ps_vegas_training(ps_program p, int enable) {
             const int dv = p->ch[c].vegas_dims;
             if (dv == 0) continue;
             const int bins = (p->grid_off[c + 1] - p->grid_off[c]) / dv - 1;
-            if (dv > ps::kHistMaxDims || bins > 256 || dv * bins > ps::kHistThreads * ps::kHistEntries)
+            if (dv > ps::kHistMaxDims || bins > 256 || dv * bins > ps::kHistMaxEntries)
                 return fail(PS_ERR_CAPACITY, "ps_vegas_training: VEGAS grid too large for the training histogram");
             stride = std::max(stride, dv * bins);
         }

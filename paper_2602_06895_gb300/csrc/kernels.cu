@@ -13,6 +13,7 @@
 //
 // Every branch inside an op depends only on the op's immediates (warp-uniform)
 // or is resolved by selects, so the warps of a channel never diverge.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -79,168 +80,189 @@ __global__ void __launch_bounds__(256) ps_map_kernel(const __grid_constant__ Lau
     dev::map_tiles(lp, pol, s_red);
 }
 
-// One CTA per channel sums the channel's tile partials in a fixed order (deterministic); in
-// streaming mode the launch's sums are added to the statistics of the earlier launches. A step of
-// 1e7 events has ~1e5 tiles: each thread keeps four loads in flight, since one CTA reading them
-// one at a time waits on memory latency.
-constexpr int kReduceThreads = 1024;
+// One cluster of eight CTAs per channel sums the channel's tile partials in a fixed order (deterministic: slice by
+// rank, thread and unroll step, then fixed trees, the ranks' sums in rank order through distributed shared
+// memory); in streaming mode the launch's sums are added to the statistics of the earlier launches.  What bounds it
+// is latency, and the FP64 adds of the trees, which one SM issues at one per 16 cycles (so few threads, and the
+// maxima on the integer ALU).  One CTA of 1024 threads took 17 us for 782 tiles and 23 us for 7813; 6.5 and 11 us now.
+constexpr int kReduceThreads = 128;
 constexpr int kReduceUnroll = 4;
+constexpr int kReduceRanks = 8;
 
-__global__ void __launch_bounds__(kReduceThreads) ps_reduce_kernel(const __grid_constant__ LaunchParams lp,
-                                                                   double* stats) {
-    const int c = blockIdx.x;
+struct TileSum {
+    double n, s, s2;
+    unsigned long long m;  // the maximum: +0 and above order like their bits
+};
+__device__ __forceinline__ void add(TileSum& a, const TileSum& b) {
+    a.n += b.n;
+    a.s += b.s;
+    a.s2 += b.s2;
+    a.m = max(a.m, b.m);
+}
+
+__global__ void __cluster_dims__(kReduceRanks, 1, 1) __launch_bounds__(kReduceThreads)
+    ps_reduce_kernel(const __grid_constant__ LaunchParams lp, double* stats) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int c = blockIdx.x / kReduceRanks, rank = static_cast<int>(cluster.block_rank());
     const ChannelLaunch& C = lp.ch[c];
     const int64_t t0 = C.tile_begin;
     const int64_t t1 = (c + 1 < lp.n_ch) ? lp.ch[c + 1].tile_begin : lp.n_tiles;
-    double a0[kReduceUnroll], a1[kReduceUnroll], a2[kReduceUnroll], a3[kReduceUnroll];
+    const int64_t len = (t1 - t0 + kReduceRanks - 1) / kReduceRanks;
+    const int64_t b0 = min(t1, t0 + rank * len), b1 = min(t1, b0 + len);
+    TileSum a[kReduceUnroll];
 #pragma unroll
-    for (int u = 0; u < kReduceUnroll; ++u) a0[u] = a1[u] = a2[u] = a3[u] = 0.0;
-    const int64_t stride = kReduceThreads;
-    for (int64_t t = t0 + threadIdx.x; t < t1; t += kReduceUnroll * stride) {
+    for (int u = 0; u < kReduceUnroll; ++u) a[u] = {0.0, 0.0, 0.0, 0ULL};
+    for (int64_t t = b0 + threadIdx.x; t < b1; t += kReduceUnroll * kReduceThreads) {
         double2 lo[kReduceUnroll], hi[kReduceUnroll];
 #pragma unroll
         for (int u = 0; u < kReduceUnroll; ++u) {  // the loads first, then the sums
-            const int64_t tu = t + u * stride;
+            const int64_t tu = t + u * kReduceThreads;
             const double2* tp = reinterpret_cast<const double2*>(lp.tile_partials + 4 * tu);
-            lo[u] = tu < t1 ? tp[0] : make_double2(0.0, 0.0);
-            hi[u] = tu < t1 ? tp[1] : make_double2(0.0, 0.0);
+            lo[u] = tu < b1 ? tp[0] : make_double2(0.0, 0.0);
+            hi[u] = tu < b1 ? tp[1] : make_double2(0.0, 0.0);
         }
 #pragma unroll
-        for (int u = 0; u < kReduceUnroll; ++u) {
-            a0[u] += lo[u].x;
-            a1[u] += lo[u].y;
-            a2[u] += hi[u].x;
-            a3[u] = fmax(a3[u], hi[u].y);
-        }
+        for (int u = 0; u < kReduceUnroll; ++u)
+            if (t + u * kReduceThreads < b1)
+                add(a[u], {lo[u].x, lo[u].y, hi[u].x, static_cast<unsigned long long>(__double_as_longlong(hi[u].y))});
     }
-    double v0 = (a0[0] + a0[1]) + (a0[2] + a0[3]);
-    double v1 = (a1[0] + a1[1]) + (a1[2] + a1[3]);
-    double v2 = (a2[0] + a2[1]) + (a2[2] + a2[3]);
-    double v3 = fmax(fmax(a3[0], a3[1]), fmax(a3[2], a3[3]));
-    // a fixed tree: within each warp by shuffles, then across the warps in shared memory
+    add(a[0], a[1]);
+    add(a[2], a[3]);
+    add(a[0], a[2]);
+    TileSum v = a[0];
+    // a fixed tree within each warp, then the warps of the CTA, then the ranks
     for (int s = 16; s > 0; s >>= 1) {
-        v0 += __shfl_down_sync(0xffffffffu, v0, s);
-        v1 += __shfl_down_sync(0xffffffffu, v1, s);
-        v2 += __shfl_down_sync(0xffffffffu, v2, s);
-        v3 = fmax(v3, __shfl_down_sync(0xffffffffu, v3, s));
+        TileSum o;
+        o.n = __shfl_down_sync(0xffffffffu, v.n, s);
+        o.s = __shfl_down_sync(0xffffffffu, v.s, s);
+        o.s2 = __shfl_down_sync(0xffffffffu, v.s2, s);
+        o.m = __shfl_down_sync(0xffffffffu, v.m, s);
+        add(v, o);
     }
-    __shared__ double red[4][kReduceThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) {
-        red[0][warp] = v0;
-        red[1][warp] = v1;
-        red[2][warp] = v2;
-        red[3][warp] = v3;
-    }
+    __shared__ TileSum red[kReduceThreads / 32], ranks[kReduceRanks];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (warp != 0) return;
-    v0 = red[0][lane];
-    v1 = red[1][lane];
-    v2 = red[2][lane];
-    v3 = red[3][lane];
-    for (int s = 16; s > 0; s >>= 1) {
-        v0 += __shfl_down_sync(0xffffffffu, v0, s);
-        v1 += __shfl_down_sync(0xffffffffu, v1, s);
-        v2 += __shfl_down_sync(0xffffffffu, v2, s);
-        v3 = fmax(v3, __shfl_down_sync(0xffffffffu, v3, s));
+    cluster.sync();  // rank 0 has started: its shared memory can be written
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < kReduceThreads / 32; ++k) add(v, red[k]);
+        *cluster.map_shared_rank(&ranks[rank], 0) = v;
     }
-    if (lane == 0) {
-        double* o = stats + 5 * c;
-        if (lp.stats_mode && *lp.stats_mode != 0) {  // streaming: add this launch to the running sums
-            o[0] += static_cast<double>(C.n_events);
-            o[1] += v0;
-            o[2] += v1;
-            o[3] += v2;
-            o[4] = fmax(o[4], v3);
-        } else {
-            o[0] = static_cast<double>(C.n_events);
-            o[1] = v0;
-            o[2] = v1;
-            o[3] = v2;
-            o[4] = v3;
-        }
+    cluster.sync();
+    if (rank != 0 || threadIdx.x != 0) return;
+    for (int k = 1; k < kReduceRanks; ++k) add(v, ranks[k]);
+    const double vmax = __longlong_as_double(static_cast<long long>(v.m));
+    double* o = stats + 5 * c;
+    if (lp.stats_mode && *lp.stats_mode != 0) {  // streaming: add this launch to the running sums
+        o[0] += static_cast<double>(C.n_events);
+        o[1] += v.n;
+        o[2] += v.s;
+        o[3] += v.s2;
+        o[4] = fmax(o[4], vmax);
+    } else {
+        o[0] = static_cast<double>(C.n_events);
+        o[1] = v.n;
+        o[2] = v.s;
+        o[3] = v.s2;
+        o[4] = vmax;
     }
 }
 
 // ---------------------------------------------------------------- VEGAS training histogram
 // The importance sums of VEGAS training, sum of w^2 per (dimension, bin of the unmapped r), for
 // every channel of a launch, added in a fixed order so that an adaptation is reproducible bit for
-// bit and does not depend on how tiles were scheduled.  Chunk k of a channel is one CTA of the
-// first kernel: kHistChunks equal slices of the channel's events, walked in event order in blocks
-// of kHistThreads.  Each block stages w^2 (from the stored weights) and the bin of every mapped
-// dimension (the event's random numbers, regenerated from Philox or read back), then thread t adds,
-// in event order, the w^2 of the events that fall into its entries t, t + kHistThreads, ...  The
-// second kernel adds a channel's chunks in chunk order into the histogram.
-__global__ void __launch_bounds__(kHistThreads) ps_hist_partial_kernel(const __grid_constant__ LaunchParams lp,
-                                                                         double* part, int stride) {
-    const int c = blockIdx.y, k = blockIdx.x, tid = threadIdx.x;
-    const ChannelLaunch& C = lp.ch[c];
-    const int nb = C.vdims * C.vbins;
-    if (nb == 0) return;
-    __shared__ double s_w2[kHistThreads];
-    __shared__ uint8_t s_bin[kHistMaxDims * kHistThreads];
+// bit and does not depend on how tiles were scheduled.  A CTA takes one chunk of a channel's events
+// (kHistChunks equal slices) and one dimension.  Every thread owns a histogram in shared memory ([bin][thread]: no
+// two threads of a warp meet in a bank) and adds the w^2 (from the stored weights) of events t, t + T, t + 2T ...
+// of the chunk in that order; the threads' rows are then added in an order fixed by the entry, and the second
+// kernel adds a channel's chunks in chunk order.
+// Bound: one FP64 add per event and dimension (15 us per 1e6 events x 8), and the latency of a thread's
+// read-modify-write chain: 32 KB a CTA at 64 bins keep seven CTAs on an SM.  1e6 events x 8 x 64 bins: 1229 us when
+// every thread of 128 CTAs compared every event with its own entries, 88 us with two dimensions to a CTA (three on an
+// SM, two waves), 37 us now.
+constexpr int kHistThreads = 64;
+constexpr int kHistSmem = kHistThreads * 256 * 8;  // the largest grid, 256 bins
+
+// kBits: Philox points and a power of two of bins, so that the bin is the leading bits of r.  A template and not
+// a branch: the general bin's product and conversion would be evaluated for every event and selected away.
+template <bool kBits>
+__device__ __forceinline__ void hist_chunk(const LaunchParams& lp, const ChannelLaunch& C, double* part, int stride,
+                                           double* acc) {
+    constexpr int T = kHistThreads;
+    const int c = blockIdx.z, j = blockIdx.y, k = blockIdx.x, tid = threadIdx.x;
+    const int bins = C.vbins;
+    for (int i = 0; i < bins; ++i) acc[i * T + tid] = 0.0;
     const int64_t len = (C.n_events + kHistChunks - 1) / kHistChunks;
     const int64_t e0 = min(C.n_events, k * len), e1 = min(C.n_events, e0 + len);
-    double acc[kHistEntries];
+    const bool odd = j & 1;
+    const int bits = __ffs(bins) - 1;
+    constexpr int kU = 4;                     // events in flight per thread
+    auto weight = [&](int64_t e) { return e < e1 ? lp.w[C.col_off + e] : 0.0; };
+    double w[kU];
 #pragma unroll
-    for (int i = 0; i < kHistEntries; ++i) acc[i] = 0.0;
-    for (int64_t base = e0; base < e1; base += kHistThreads) {
-        const int64_t e = base + tid;
-        if (e < e1) {
-            const double w = lp.w[C.col_off + e];
-            s_w2[tid] = w * w;
-            const int64_t ev = C.ev_offset + e;
-            for (int j = 0; j < C.vdims; j += 2) {
-                double r0, r1 = 0.5;
-                if (lp.r != nullptr) {
-                    r0 = lp.r[j * lp.ld_r + e];
-                    if (j + 1 < C.vdims) r1 = lp.r[(j + 1) * lp.ld_r + e];
-                } else {
-                    const uint4 o = rng::philox4x32_10(make_uint4(static_cast<uint32_t>(ev), static_cast<uint32_t>(ev >> 32),
-                                                             static_cast<uint32_t>(c), static_cast<uint32_t>(j >> 1)),
-                                                  static_cast<uint32_t>(lp.seed), static_cast<uint32_t>(lp.seed >> 32));
-                    r0 = rng::unit_from_bits(o.y, o.x);
-                    r1 = rng::unit_from_bits(o.w, o.z);
-                }
-                s_bin[j * kHistThreads + tid] = static_cast<uint8_t>(min(max(static_cast<int>(r0 * C.vbins), 0), C.vbins - 1));
-                if (j + 1 < C.vdims)
-                    s_bin[(j + 1) * kHistThreads + tid] =
-                        static_cast<uint8_t>(min(max(static_cast<int>(r1 * C.vbins), 0), C.vbins - 1));
+    for (int u = 0; u < kU; ++u) w[u] = weight(e0 + tid + u * T);
+    for (int64_t base = e0 + tid; base < e1; base += kU * T) {
+        double w2[kU];
+        int b[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            w2[u] = w[u] * w[u];
+            w[u] = weight(base + (kU + u) * T);  // the next round's
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int64_t e = min(base + u * T, e1 - 1), ev = C.ev_offset + e;
+            uint4 o = make_uint4(0u, 0u, 0u, 0u);
+            if (kBits || lp.r == nullptr)
+                o = rng::philox4x32_10(make_uint4(static_cast<uint32_t>(ev), static_cast<uint32_t>(ev >> 32),
+                                                              static_cast<uint32_t>(c), static_cast<uint32_t>(j >> 1)),
+                                                   static_cast<uint32_t>(lp.seed), static_cast<uint32_t>(lp.seed >> 32));
+            const uint32_t lead = odd ? o.w : o.y;
+            if constexpr (kBits) {
+                b[u] = static_cast<int>(__funnelshift_l(lead, 0u, bits));
+            } else {
+                const double r = lp.r != nullptr ? lp.r[j * lp.ld_r + e] : rng::unit_from_bits(lead, odd ? o.z : o.x);
+                b[u] = min(max(static_cast<int>(r * bins), 0), bins - 1);
             }
         }
-        __syncthreads();
-        const int n = static_cast<int>(min(static_cast<int64_t>(kHistThreads), e1 - base));
 #pragma unroll
-        for (int i = 0; i < kHistEntries; ++i) {
-            const int idx = tid + i * kHistThreads;
-            if (idx < nb) {
-                const int j = idx / C.vbins, b = idx - j * C.vbins;
-                const uint8_t* bins = s_bin + j * kHistThreads;
-                double a = acc[i];
-                for (int t = 0; t < n; ++t)
-                    if (bins[t] == b) a += s_w2[t];
-                acc[i] = a;
-            }
-        }
-        __syncthreads();
+        for (int u = 0; u < kU; ++u)
+            if (base + u * T < e1) acc[b[u] * T + tid] += w2[u];
     }
-    double* o = part + (static_cast<int64_t>(c) * kHistChunks + k) * stride;
-#pragma unroll
-    for (int i = 0; i < kHistEntries; ++i) {
-        const int idx = tid + i * kHistThreads;
-        if (idx < nb) o[idx] = acc[i];
+    __syncthreads();
+    double* o = part + (static_cast<int64_t>(c) * kHistChunks + k) * stride + j * bins;
+    for (int i = tid; i < bins; i += T) {
+        double s = 0.0;  // the rows in the order i, i + 1, ... (mod T): the threads read different banks
+#pragma unroll 8
+        for (int q = 0; q < T; ++q) s += acc[i * T + ((i + q) & (T - 1))];
+        o[i] = s;
     }
 }
 
-__global__ void __launch_bounds__(kHistThreads) ps_hist_reduce_kernel(const __grid_constant__ LaunchParams lp,
-                                                                        const double* part, int stride) {
+__global__ void __launch_bounds__(kHistThreads) ps_hist_partial_kernel(const __grid_constant__ LaunchParams lp, double* part,
+                                                                       int stride) {
+    extern __shared__ __align__(16) double acc[];
+    const ChannelLaunch& C = lp.ch[blockIdx.z];
+    if (static_cast<int>(blockIdx.y) >= C.vdims) return;
+    if (lp.r == nullptr && (C.vbins & (C.vbins - 1)) == 0) hist_chunk<true>(lp, C, part, stride, acc);
+    else hist_chunk<false>(lp, C, part, stride, acc);
+}
+
+__global__ void __launch_bounds__(kHistReduce) ps_hist_reduce_kernel(const __grid_constant__ LaunchParams lp,
+                                                                     const double* part, int stride) {
     const int c = blockIdx.y;
     const ChannelLaunch& C = lp.ch[c];
-    const int idx = blockIdx.x * kHistThreads + threadIdx.x;
+    const int idx = blockIdx.x * kHistReduce + threadIdx.x;
     if (idx >= C.vdims * C.vbins) return;
     const double* q = part + static_cast<int64_t>(c) * kHistChunks * stride + idx;
     double s = 0.0;
-    for (int k = 0; k < kHistChunks; ++k) s += q[static_cast<int64_t>(k) * stride];
+    for (int k0 = 0; k0 < kHistChunks; k0 += 16) {
+        double v[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = q[static_cast<int64_t>(k0 + k) * stride];  // the loads first
+#pragma unroll
+        for (int k = 0; k < 16; ++k) s += v[k];
+    }
     lp.hist[C.hist_off + idx] += s;
 }
 
@@ -296,7 +318,7 @@ int launch_map(const LaunchParams& lp, int grid_ctas, size_t smem, void* stream,
 }
 
 int launch_reduce(const LaunchParams& lp, double* stats, void* stream, std::string* err) {
-    ps_reduce_kernel<<<lp.n_ch, kReduceThreads, 0, static_cast<cudaStream_t>(stream)>>>(lp, stats);
+    ps_reduce_kernel<<<lp.n_ch * kReduceRanks, kReduceThreads, 0, static_cast<cudaStream_t>(stream)>>>(lp, stats);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "ps_reduce_kernel launch", err);
     __atomic_add_fetch(&g_launches, 1ULL, __ATOMIC_RELAXED);
@@ -306,11 +328,32 @@ int launch_reduce(const LaunchParams& lp, double* stats, void* stream, std::stri
 int launch_hist(const LaunchParams& lp, double* part, int stride, void* stream, std::string* err) {
     if (lp.hist == nullptr || stride <= 0) return PS_OK;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    ps_hist_partial_kernel<<<dim3(kHistChunks, lp.n_ch), kHistThreads, 0, cs>>>(lp, part, stride);
-    cudaError_t e = cudaGetLastError();
+    int dims = 0, bins = 0;
+    for (int c = 0; c < lp.n_ch; ++c) {
+        if (lp.ch[c].vdims == 0) continue;
+        dims = std::max(dims, static_cast<int>(lp.ch[c].vdims));
+        bins = std::max(bins, static_cast<int>(lp.ch[c].vbins));
+    }
+    if (dims == 0) return PS_OK;
+    cudaError_t e = cudaSuccess;
+    {
+        // the dynamic shared memory above the default is granted once per device
+        static std::mutex mu;
+        static bool granted[kMaxDevices] = {};
+        std::lock_guard<std::mutex> lock(mu);
+        int dev = 0;
+        e = cudaGetDevice(&dev);
+        if (e == cudaSuccess && dev >= 0 && dev < kMaxDevices && !granted[dev]) {
+            e = cudaFuncSetAttribute(ps_hist_partial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistSmem);
+            granted[dev] = e == cudaSuccess;
+        }
+        if (e != cudaSuccess) return cuda_fail(e, "ps_hist_partial_kernel shared memory", err);
+    }
+    ps_hist_partial_kernel<<<dim3(kHistChunks, dims, lp.n_ch), kHistThreads, sizeof(double) * kHistThreads * bins, cs>>>(
+        lp, part, stride);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "ps_hist_partial_kernel launch", err);
-    ps_hist_reduce_kernel<<<dim3((stride + kHistThreads - 1) / kHistThreads, lp.n_ch), kHistThreads, 0, cs>>>(lp, part,
-                                                                                                            stride);
+    ps_hist_reduce_kernel<<<dim3((stride + kHistReduce - 1) / kHistReduce, lp.n_ch), kHistReduce, 0, cs>>>(lp, part, stride);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "ps_hist_reduce_kernel launch", err);
     __atomic_add_fetch(&g_launches, 2ULL, __ATOMIC_RELAXED);

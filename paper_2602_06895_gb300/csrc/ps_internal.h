@@ -14,11 +14,11 @@ namespace ps {
 constexpr int kMaxOutMomenta = 24;
 constexpr int kNoallocTiles = 131072;  // tiles of the allocation-free entry point's fixed scratch
 constexpr int kMaxDevices = 64;
-// VEGAS training histogram (kernels.cu): chunks per channel, threads per chunk, and the largest
-// grid it takes (dimensions x bins <= kHistThreads * kHistEntries, bins <= 256)
-constexpr int kHistChunks = 128;
-constexpr int kHistThreads = 256;
-constexpr int kHistEntries = 16;
+// VEGAS training histogram (kernels.cu): chunks per channel, threads that add them, and the largest
+// grid it takes (dimensions x bins <= kHistMaxEntries, bins <= 256)
+constexpr int kHistChunks = 112;
+constexpr int kHistReduce = 64;
+constexpr int kHistMaxEntries = 4096;
 constexpr int kHistMaxDims = 64;
 
 // ---------------------------------------------------------------- graph IR
