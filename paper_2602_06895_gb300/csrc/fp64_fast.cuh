@@ -362,6 +362,54 @@ __device__ __forceinline__ double root1p(double p, int n) {
     return __dadd_rn(r, -fma(c, widen_or_zero(t), c));
 }
 
+// The exponent w = 1 - nu of a power law, near 1/n for an integer n: n w = 1 - eta.
+struct WholePower {
+    int n;
+    double nd;  // n
+    float eta;
+    bool ok;    // 2 <= n <= kMaxPower and |eta| < 1e-13
+};
+__device__ __forceinline__ WholePower whole_power(double w, bool constant) {  // constant: of a compiled channel, folds
+    WholePower p;
+    const float wf = constant ? static_cast<float>(w) : narrow(w);
+    const float nf = rintf(constant ? 1.0f / wf : rcp_approx(wf));
+    const bool near = wf > 0.15f && wf < 0.55f && fabsf(fmaf(-nf, wf, 1.0f)) < 1e-6f;
+    p.nd = constant ? static_cast<double>(nf) : widen(near ? nf : 1.0f);
+    const double eta = fma(-p.nd, w, 1.0);
+    p.eta = constant ? static_cast<float>(eta) : narrow(eta);
+    p.n = static_cast<int>(nf);
+    p.ok = near && fabsf(p.eta) < 1e-13f;
+    return p;
+}
+__device__ __forceinline__ bool root_arg(double p) { return hi32(p) - 0x3C300000u < 0x0A000000u; }  // [2^-60, 2^100)
+// (1 + p)^w - 1, root_arg(p): (1 + p)^-eta to first order moves p by -eta (1 + p) log(1 + p)
+__device__ __forceinline__ double power_root(double p, const WholePower& k) {
+    const float pf = narrow(p);
+    const float dp = k.eta * (1.0f + pf) * (0.693147181f * lg2_approx(1.0f + pf));
+    return root1p(k.eta != 0.0f ? __dadd_rn(p, -widen_or_zero(dp)) : p, k.n);
+}
+
+// ---------------------------------------------------------------- powers
+// log x of a positive normal x as a head on the grid of 2^-41 and a rest (below 2^-8) good to 2^-61
+__device__ __forceinline__ void log_pair(double x, double& head, double& rest) {
+    const uint32_t hi = hi32(x);
+    const int j = static_cast<int>(((hi & 0xFFFFFu) + 0x800u) >> 12);
+    const double m = from32((hi & 0xFFFFFu) | 0x3FF00000u, lo32(x));
+    const double2 t = __ldg(reinterpret_cast<const double2*>(kLogTab) + j);
+    const double Ed = widen_int(__int_as_float(0x4B400000 + static_cast<int>(hi >> 20) - 1023) - 12582912.0f);
+    const double r = fma(m, widen(__ldg(&kLogInv[j])), -1.0);
+    const float rf = narrow(r);
+    const double g = widen(fmaf(rf, fmaf(rf, fmaf(rf, 1.0f / 7.0f, -1.0f / 6.0f), 0.2f), -0.25f));
+    head = fma(Ed, kLn2Hi, t.x);
+    rest = __dadd_rn(fma(Ed, kLn2Lo, t.y), fma(__dmul_rn(r, r), fma(r, fma(r, g, 1.0 / 3.0), -0.5), r));
+}
+// exp(a (head + rest)): the product as a pair
+__device__ __forceinline__ double exp_of(double a, double head, double rest) {
+    const double v = __dmul_rn(a, head), w = fma(a, rest, fma(a, head, -v));
+    const double s = __dadd_rn(v, w);
+    return exp(s, __dadd_rn(w, -__dadd_rn(s, -v)));
+}
+
 }  // namespace fast
 }  // namespace dev
 }  // namespace ps

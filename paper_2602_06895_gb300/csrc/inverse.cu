@@ -30,25 +30,39 @@ using dev::P4;
 
 constexpr int kMaxLeg = kMaxOutMomenta + 2;
 
+namespace fast = dev::fast;
+
 // Both inverse maps: where rounding has collapsed the range to a point every r maps to it, and 0 is
 // returned (the quotients below would be 0/0 or infinite).
-// inverse power-law map (anchored as the forward map)
-__device__ __forceinline__ double inv_nu(double x, double m, double nu, double xmin, double xmax, double a) {
-    const double m2 = (m > 0.0) ? m * m : -a;
-    const double lo = xmin - m2, hi = xmax - m2;
-    if (xmax <= xmin) return 0.0;
-    const double L = log1p((xmax - xmin) / lo);
-    if (nu == 1.0) return log1p((x - xmin) / lo) / L;
-    const double w = 1.0 - nu;
-    if (nu < 1.0) return expm1(w * log1p((x - xmin) / lo)) / expm1(w * L);
-    return 1.0 - expm1(w * log((x - m2) / hi)) / expm1(-w * L);
+// (comparisons on the bits here and below: the FP64 pipe that bounds the kernel would execute them)
+__device__ __forceinline__ bool empty_range(double xmin, double xmax) {  // x_max <= x_min for bounds >= 0
+    return dev::dbits(xmax) <= dev::dbits(xmin);
 }
 
-// inverse Breit-Wigner map: the angle measured from the nearer end of the range
+// inverse power-law map (anchored as the forward map; by roots where 1/(1 - nu) is an integer, as there: 31 FP64
+// instructions where the logarithms and exponentials take 47 and CUDA's took 130)
+__device__ __forceinline__ double inv_nu(double x, double m, double nu, double xmin, double xmax, double a) {
+    const double m2 = dev::pos_bits(m) ? m * m : -a;
+    const double lo = xmin - m2, hi = xmax - m2;
+    if (empty_range(xmin, xmax)) return 0.0;
+    const double p = fast::div(xmax - xmin, lo), q = fast::div(x - xmin, lo);
+    if (dev::dbits(nu) == dev::dbits(1.0)) return fast::div(fast::log1p(q), fast::log1p(p));
+    const double w = 1.0 - nu;
+    if (dev::dbits(nu) < dev::dbits(1.0)) {
+        const fast::WholePower k = fast::whole_power(w, false);
+        if (k.ok && fast::root_arg(p) && fast::root_arg(q)) return fast::div(fast::power_root(q, k), fast::power_root(p, k));
+        return fast::div(fast::expm1(w * fast::log1p(q)), fast::expm1(w * fast::log1p(p)));
+    }
+    return 1.0 - fast::div(fast::expm1(w * fast::log(fast::div(x - m2, hi))), fast::expm1(-w * fast::log1p(p)));
+}
+
+// inverse Breit-Wigner map: the angle measured from the nearer end of the range.  With CUDA's functions: far above a
+// narrow resonance r is within 1e-8 of 1, one ulp of it moves the density there by 1e-8, and this is the rounding
+// that earlier densities were computed with.
 __device__ __forceinline__ double inv_bw(double x, double M, double G, double xmin, double xmax) {
     const double mg = M * G, m2 = M * M;
     const double a = (xmin - m2) / mg, b = (xmax - m2) / mg;
-    if (xmax <= xmin) return 0.0;
+    if (empty_range(xmin, xmax)) return 0.0;
     const double D = atan2((xmax - xmin) / mg, fma(a, b, 1.0));
     const double t = (x - m2) / mg;
     if (x - xmin <= xmax - x) return atan2((x - xmin) / mg, fma(a, t, 1.0)) / D;
@@ -57,12 +71,20 @@ __device__ __forceinline__ double inv_bw(double x, double M, double G, double xm
 
 __device__ __forceinline__ double inv_invariant(double x, double M, double G, double nu, double xmin, double xmax,
                                                 double a) {
-    return G > 0.0 ? inv_bw(x, M, G, xmin, xmax) : inv_nu(x, M, nu, xmin, xmax, a);
+    return dev::pos_bits(G) ? inv_bw(x, M, G, xmin, xmax) : inv_nu(x, M, nu, xmin, xmax, a);
+}
+
+// p into the rest frame of q of mass m (1/m given).  Quotients and not products with reciprocals here and in the
+// kernel: their extra rounding raised the error of the densities by 13%, at 5% of the kernel's time.
+__device__ __forceinline__ P4 to_rest(const P4& p, const P4& q, double m, double inv_m) {
+    const double qp = q.x * p.x + q.y * p.y + q.z * p.z;
+    const double c = fma(-p.e, inv_m, fast::div(qp, m * (q.e + m)));
+    return {(q.e * p.e - qp) * inv_m, p.x + q.x * c, p.y + q.y * c, p.z + q.z * c};
 }
 
 __device__ __forceinline__ double unit_phi(double y, double x) {
-    double ph = atan2(y, x) / (2.0 * kPi);
-    return ph < 0.0 ? ph + 1.0 : ph;
+    const double ph = fast::atan2(fabs(y), x) * (0.5 / kPi);
+    return dev::dbits(y) < 0 && !dev::is_zero(y) ? 1.0 - ph : ph;
 }
 
 __device__ __forceinline__ double vegas_inv(double rp, const double* e, int N) {
@@ -90,25 +112,28 @@ __global__ void __launch_bounds__(128) ps_inverse_kernel(const __grid_constant__
 
     // SDE propagator product from the lab momenta (q_k = p_a - legs for t-channel propagators)
     if (Pout) {
-        double prod = 1.0;
+        double den = 1.0, prod = 1.0;
         for (int k = 0; k < P.n_prop; ++k) {
             P4 s = P.pkind[k] == 1 ? q[0] : P4{0.0, 0.0, 0.0, 0.0};
             const double sg = P.pkind[k] == 1 ? -1.0 : 1.0;
             for (int i = 0; i < n; ++i)
                 if (P.pmask[k] & (1u << i)) s = {s.e + sg * q[2 + i].e, s.x + sg * q[2 + i].x, s.y + sg * q[2 + i].y,
                                                  s.z + sg * q[2 + i].z};
-            const double inv = dev::p4_sq(s);
-            const double dd = inv - P.pM[k] * P.pM[k];
-            prod *= P.pkind[k] == 1 ? 1.0 / (dd * dd) : 1.0 / (dd * dd + P.pM[k] * P.pM[k] * P.pG[k] * P.pG[k]);
+            const double dd = dev::p4_sq(s) - P.pM[k] * P.pM[k], mg = P.pM[k] * P.pG[k];
+            den *= P.pkind[k] == 1 ? dd * dd : fma(dd, dd, mg * mg);
+            if (den > 1e200) {  // keep the running product in range
+                prod = fast::slow_div(prod, den);
+                den = 1.0;
+            }
         }
-        Pout[b] = prod;
+        Pout[b] = fast::div(prod, den);
     }
 
     // partonic frame (light-cone form of the inverse longitudinal boost)
     if (P.hadronic && P.lab_frame) {
-        const double rho = sqrt(x1 / x2);
+        const double rho = fast::sqrt(fast::div(x1, x2));
         for (int i = 0; i < n + 2; ++i) {
-            const double plus = (q[i].e + q[i].z) / rho, minus = rho * (q[i].e - q[i].z);
+            const double plus = fast::div(q[i].e + q[i].z, rho), minus = rho * (q[i].e - q[i].z);
             q[i].e = 0.5 * (plus + minus);
             q[i].z = 0.5 * (plus - minus);
         }
@@ -125,11 +150,11 @@ __global__ void __launch_bounds__(128) ps_inverse_kernel(const __grid_constant__
             ml[i] = P.node[j].mass;
             if (any_decay) {
                 const P4 p = q[2 + i];
-                const double a = sqrt(p.x * p.x + p.y * p.y + p.z * p.z);
+                const double a = fast::sqrt(p.x * p.x + p.y * p.y + p.z * p.z);
                 ap[i] = a;
-                nx[i] = p.x / a;
-                ny[i] = p.y / a;
-                nz[i] = p.z / a;
+                nx[i] = fast::div(p.x, a);
+                ny[i] = fast::div(p.y, a);
+                nz[i] = fast::div(p.z, a);
             }
         }
     P4 pn[kInvNodes];
@@ -152,36 +177,40 @@ __global__ void __launch_bounds__(128) ps_inverse_kernel(const __grid_constant__
                 if (!(mask & (1u << k))) continue;
                 const double dx = nx[i] - nx[k], dy = ny[i] - ny[k], dz = nz[i] - nz[k];
                 const double mi2 = ml[i] * ml[i], mk2 = ml[k] * ml[k];
-                s2 += 2.0 * (mi2 * ap[k] * ap[k] + mk2 * ap[i] * ap[i] + mi2 * mk2) /
-                          (q[2 + i].e * q[2 + k].e + ap[i] * ap[k]) +
-                      ap[i] * ap[k] * (dx * dx + dy * dy + dz * dz);
+                s2 += ap[i] * ap[k] * (dx * dx + dy * dy + dz * dz);
+                if (!(dev::is_zero(mi2) && dev::is_zero(mk2)))
+                    s2 += fast::div(2.0 * (mi2 * ap[k] * ap[k] + mk2 * ap[i] * ap[i] + mi2 * mk2),
+                                    q[2 + i].e * q[2 + k].e + ap[i] * ap[k]);
             }
         }
         pn[j] = acc;
         s[j] = s2;
     }
-    auto leg_mass = [&](int j) { return P.node[j].kind == PS_NODE_LEAF ? P.node[j].mass : sqrt(s[j]); };
+    double root[kInvNodes];  // sqrt(s) of the decay nodes
+    auto leg_mass = [&](int j) { return P.node[j].kind == PS_NODE_LEAF ? P.node[j].mass : root[j]; };
 
     double shat;
     if (P.hadronic) {
         shat = x1 * x2 * P.S;
         r[P.d_shat * ldr + b] = inv_invariant(shat, P.shat_M, P.shat_G, P.shat_nu, P.mleaf * P.mleaf, P.S, P.a);
-        r[P.d_x * ldr + b] = log(x1) / log(shat / P.S);
+        r[P.d_x * ldr + b] = fast::div(fast::log(x1), fast::log(fast::div(shat, P.S)));
     } else {
         shat = P.sqrt_s * P.sqrt_s;
     }
     s[0] = shat;
+    for (int j = 0; j < P.n_nodes; ++j)
+        if (j == 0 || P.node[j].kind == PS_NODE_DECAY) root[j] = fast::sqrt(s[j]);
 
     // s-channel invariants with the forward's bounds
     for (int i = 0; i < P.n_sorder; ++i) {
         const int j = P.sorder[i];
         double mlo = P.lo_c[i];
-        for (int k = P.lo_beg[i]; k < P.off_beg[i]; ++k) mlo += sqrt(s[P.ids[k]]);
+        for (int k = P.lo_beg[i]; k < P.off_beg[i]; ++k) mlo += root[P.ids[k]];
         double off = P.off_c[i];
-        for (int k = P.off_beg[i]; k < P.lo_beg[i + 1]; ++k) off += sqrt(s[P.ids[k]]);
+        for (int k = P.off_beg[i]; k < P.lo_beg[i + 1]; ++k) off += root[P.ids[k]];
         const int top = P.top[i];
-        const double mtop = (top == 0 && !P.hadronic) ? P.sqrt_s : sqrt(s[top]);
-        const double mhi = fmax(mtop - off, mlo);
+        const double mtop = (top == 0 && !P.hadronic) ? P.sqrt_s : root[top];
+        const double mhi = dev::fmax_bits(mtop - off, mlo);
         const InvNode& nd = P.node[j];
         r[P.d_s[j] * ldr + b] = inv_invariant(s[j], nd.M, nd.G, nd.nu, mlo * mlo, mhi * mhi, P.a);
     }
@@ -190,8 +219,9 @@ __global__ void __launch_bounds__(128) ps_inverse_kernel(const __grid_constant__
     const int kappa = P.kappa;
     if (kappa > 0) {
         const InvNode& root = P.node[0];
-        double sts[kInvLegs + 1];
+        double sts[kInvLegs + 1], rts[kInvLegs + 1], irs[kInvLegs + 1];  // the block invariants, roots and their reciprocals
         sts[0] = shat;
+        rts[0] = fast::sqrt_rcp(shat, irs[0]);
         int l2 = 0, r2 = kappa;
         for (int i = 1; i < kappa; ++i) {
             if (P.side[i] == 0) ++l2;
@@ -204,11 +234,12 @@ __global__ void __launch_bounds__(128) ps_inverse_kernel(const __grid_constant__
             }
             sts[i] = dev::p4_sq(c);
             const double mi = leg_mass(root.child[P.order[i]]);
-            const double mx = fmax(sqrt(sts[i - 1]) - mi, 0.0);
+            rts[i] = fast::sqrt_rcp(sts[i], irs[i]);
+            const double mx = dev::fmax_bits(rts[i - 1] - mi, 0.0);
             const double smin = msum * msum;
-            r[P.d_ts[i] * ldr + b] = inv_nu(sts[i], 0.0, P.ts_nu, smin, fmax(mx * mx, smin), P.a);
+            r[P.d_ts[i] * ldr + b] = inv_nu(sts[i], 0.0, P.ts_nu, smin, dev::fmax_bits(mx * mx, smin), P.a);
         }
-        const double e0 = 0.5 * sqrt(shat);
+        const double e0 = 0.5 * rts[0];
         P4 pA{e0, 0.0, 0.0, e0}, pB{e0, 0.0, 0.0, -e0};
         double mA2 = 0.0, mB2 = 0.0, scur = shat;
         for (int i = 1; i <= kappa; ++i) {
@@ -223,29 +254,28 @@ __global__ void __launch_bounds__(128) ps_inverse_kernel(const __grid_constant__
             } else if (P.side[i] == 0) {
                 const int l1 = root.child[P.order[i]];
                 m1 = leg_mass(l1);
-                m2 = sqrt(sts[i]);
+                m2 = rts[i];
                 q1 = pn[l1];
                 q2 = dev::p4_sub(dev::p4_add(pA, pB), q1);
             } else {
                 const int l1 = root.child[P.order[i]];
-                m1 = sqrt(sts[i]);
+                m1 = rts[i];
                 m2 = leg_mass(l1);
                 q2 = pn[l1];
                 q1 = dev::p4_sub(dev::p4_add(pA, pB), q2);
             }
             const double tabs = -dev::p4_sq(dev::p4_sub(pA, q1));
-            double tmin, tmax, Bt;
-            dev::t_range(scur, mA2, mB2, m1, m2, tmin, tmax, Bt);
-            const double tlo = fmax(tmin, 0.0), thi = fmax(tmax, tlo);
+            const dev::TRange tr = dev::t_range_fast(scur, mA2, mB2, m1, m2);
+            const double tlo = dev::fmax_bits(tr.lo, 0.0), thi = dev::fmax_bits(tr.hi, tlo);
             r[P.d_tt[i] * ldr + b] = inv_nu(tabs, 0.0, P.t_nu, tlo, thi, P.a);
             // azimuth of q1 about the direction of pA in the block rest frame
             const P4 p0 = dev::p4_add(pA, pB);
-            const double m0 = sqrt(scur);
-            const P4 pAs = dev::boost_in(pA, p0, m0), q1s = dev::boost_in(q1, p0, m0);
-            const double pt = sqrt(pAs.x * pAs.x + pAs.y * pAs.y);
-            const double pp = sqrt(pt * pt + pAs.z * pAs.z);
-            const double cA = pAs.z / pp, sA = pt / pp;
-            const double cpA = pt > 0.0 ? pAs.x / pt : 1.0, spA = pt > 0.0 ? pAs.y / pt : 0.0;
+            const P4 pAs = to_rest(pA, p0, rts[i - 1], irs[i - 1]), q1s = to_rest(q1, p0, rts[i - 1], irs[i - 1]);
+            const double pt = fast::sqrt(pAs.x * pAs.x + pAs.y * pAs.y);
+            const double pp = fast::sqrt(pt * pt + pAs.z * pAs.z);
+            const double cA = fast::div(pAs.z, pp), sA = fast::div(pt, pp);
+            const bool off_axis = dev::pos_bits(pt);
+            const double cpA = off_axis ? fast::div(pAs.x, pt) : 1.0, spA = off_axis ? fast::div(pAs.y, pt) : 0.0;
             const double v1 = cpA * q1s.x + spA * q1s.y;
             const double v2 = -spA * q1s.x + cpA * q1s.y;
             r[P.d_tphi[i] * ldr + b] = unit_phi(v2, cA * v1 - sA * q1s.z);
@@ -266,11 +296,12 @@ __global__ void __launch_bounds__(128) ps_inverse_kernel(const __grid_constant__
     for (int i = 0; i < P.n_pre; ++i) {
         const int j = P.pre[i];
         const int c1 = P.node[j].child[0];
-        const P4 qq = j == 0 ? pn[c1] : dev::boost_in(pn[c1], pn[j], sqrt(s[j]));
+        const P4 qq = j == 0 ? pn[c1] : to_rest(pn[c1], pn[j], root[j], fast::rcp(root[j]));
         const double pt2 = qq.x * qq.x + qq.y * qq.y;
-        const double pa = sqrt(pt2 + qq.z * qq.z);
+        const double pa = fast::sqrt(pt2 + qq.z * qq.z);
         // r_theta = (1 + cos theta)/2 in the sin^2(theta/2) form near the poles
-        const double rth = qq.z >= 0.0 ? 1.0 - 0.5 * (pt2 / (pa * (pa + qq.z))) : 0.5 * (pt2 / (pa * (pa - qq.z)));
+        const double h = 0.5 * fast::div(pt2, pa * (pa + fabs(qq.z)));
+        const double rth = dev::dbits(qq.z) >= 0 || dev::is_zero(qq.z) ? 1.0 - h : h;
         r[P.d_dth[j] * ldr + b] = rth;
         r[P.d_dphi[j] * ldr + b] = unit_phi(qq.y, qq.x);
     }
@@ -283,6 +314,27 @@ struct GlobalArgs {
     double alpha[kMaxChannels];
 };
 
+// (x1 x2)^pa ((1 - x1)(1 - x2))^pb: one exponential of the sum of the logarithms as pairs, and for pb = 1, 2, 3
+// products (38 FP64 instructions where four powers take 330; relative error below 4e-16 either way).  Outside
+// 0 < x < 1 and for infinite or NaN exponents: the powers.
+__device__ __forceinline__ double pdf_pair(double x1, double x2, double pa, double pb) {
+    auto inside = [](double x) { return fast::hi32(x) - 0x00100000u < 0x3FE00000u; };  // positive, normal, below 1
+    if (!(inside(x1) && inside(x2) && fabs(pa) < 1e3 && fabs(pb) < 1e3))
+        return pow(x1, pa) * pow(1.0 - x1, pb) * pow(x2, pa) * pow(1.0 - x2, pb);
+    double h1, l1, h2, l2;
+    fast::log_pair(x1, h1, l1);
+    fast::log_pair(x2, h2, l2);
+    const double f = fast::exp_of(pa, h1 + h2, l1 + l2);
+    const double y1 = 1.0 - x1, y2 = 1.0 - x2;
+    if (pb == 3.0) return f * (y1 * y1 * y1) * (y2 * y2 * y2);
+    if (pb == 2.0) return f * (y1 * y1) * (y2 * y2);
+    if (pb == 1.0) return f * y1 * y2;
+    if (pb == 0.0) return f;
+    fast::log_pair(y1, h1, l1);
+    fast::log_pair(y2, h2, l2);
+    return f * fast::exp_of(pb, h1 + h2, l1 + l2);
+}
+
 // w = f / sum_j alpha_j g_j with g_j = 1 / J_j (J_j = 0: outside channel j, no density); f is
 // the given integrand, or pdf(x1) pdf(x2) sum_j P_j (the SDE propagator sum) when f is null.
 __global__ void ps_global_weight_kernel(const __grid_constant__ GlobalArgs A, int64_t batch, const double* J,
@@ -293,7 +345,7 @@ __global__ void ps_global_weight_kernel(const __grid_constant__ GlobalArgs A, in
     double g = 0.0;
     for (int j = 0; j < A.n_ch; ++j) {
         const double Jj = J[j * ldj + b];
-        if (Jj > 0.0) g += A.alpha[j] / Jj;
+        if (dev::pos_bits(Jj)) g += fast::div(A.alpha[j], Jj);
     }
     double fv;
     if (f) {
@@ -302,9 +354,9 @@ __global__ void ps_global_weight_kernel(const __grid_constant__ GlobalArgs A, in
         double ps = 0.0;
         for (int j = 0; j < A.n_ch; ++j) ps += Pp[j * ldp + b];
         fv = ps;
-        if (x1) fv *= pow(x1[b], pa) * pow(1.0 - x1[b], pb) * pow(x2[b], pa) * pow(1.0 - x2[b], pb);
+        if (x1) fv *= pdf_pair(x1[b], x2[b], pa, pb);
     }
-    w[b] = g > 0.0 ? fv / g : 0.0;
+    w[b] = g > 0.0 ? fast::div(fv, g) : 0.0;
 }
 
 }  // namespace inv

@@ -132,32 +132,22 @@ __device__ __forceinline__ bool map_nu(double r, double m, double nu, double xmi
     const double range = sub_z(xmax, xmin);
     const double p = have_L && const_nu ? range / lo : fast::div(range, lo);
     const double w = __dadd_rn(1.0, -nu);
-    const float wf = const_nu ? static_cast<float>(w) : fast::narrow(w);
-    const float nf = rintf(const_nu ? 1.0f / wf : fast::rcp_approx(wf));
-    const bool near = wf > 0.15f && wf < 0.55f && fabsf(fmaf(-nf, wf, 1.0f)) < 1e-6f;
-    const double nd = const_nu ? static_cast<double>(nf) : fast::widen(near ? nf : 1.0f);
-    const double eta = fma(-nd, w, 1.0);
-    const float ef = const_nu ? static_cast<float>(eta) : fast::narrow(eta);
-    const bool whole = near && fabsf(ef) < 1e-13f;
-    const bool in_range = fast::hi32(p) - 0x3C300000u < 0x0A000000u;
-    if (whole && (const_nu || in_range)) {
-        const int n = static_cast<int>(nf);
-        const float pf = fast::narrow(p);
-        // 1 + p to the power -eta: p' = p - eta (1 + p) log(1 + p)
-        const float dp = ef * (1.0f + pf) * (0.693147181f * fast::lg2_approx(1.0f + pf));
-        const double rho = fast::root1p(ef != 0.0f ? __dadd_rn(p, -fast::widen_or_zero(dp)) : p, n);
+    const fast::WholePower k = fast::whole_power(w, const_nu);
+    const bool in_range = fast::root_arg(p);
+    if (k.ok && (const_nu || in_range)) {
+        const double rho = fast::power_root(p, k);
         const double z = __dmul_rn(r, rho), u = __dadd_rn(1.0, z);
         double s_prev, s_n;
-        fast::geometric(u, n, s_prev, s_n);
+        fast::geometric(u, k.n, s_prev, s_n);
         double e = __dmul_rn(z, s_n), pw = fma(z, s_prev, 1.0);  // u^n - 1 and u^(n-1)
-        if (ef != 0.0f) {
+        if (k.eta != 0.0f) {  // (1 + z)^(n eta) to first order
             const float uf = fast::narrow(u), pwf = fast::narrow(pw);
-            const float d = pwf * (nf * ef) * (0.693147181f * fast::lg2_approx(uf));
+            const float d = pwf * (static_cast<float>(k.n) * k.eta) * (0.693147181f * fast::lg2_approx(uf));
             e = __dadd_rn(e, fast::widen_or_zero(d * uf));
             pw = __dadd_rn(pw, fast::widen_or_zero(d));
         }
         x = fma(lo, e, xmin);
-        jac = __dmul_rn(__dmul_rn(__dmul_rn(lo, rho), pw), fma(nd, eta, nd));  // 1/w = n (1 + eta)
+        jac = __dmul_rn(__dmul_rn(__dmul_rn(lo, rho), pw), fma(k.nd, fma(-k.nd, w, 1.0), k.nd));  // 1/w = n (1 + eta)
         if (const_nu && __builtin_expect(!in_range, 0)) {
             const NuOut o = map_nu_far(r, nu, xmin, lo, hi, m2, p);
             x = o.x;
