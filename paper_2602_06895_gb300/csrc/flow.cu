@@ -283,7 +283,13 @@ struct Args {
     float* rowsum;     // kAtomic with A unit-stride along k: row sums of A (bias gradient), atomic
 };
 
-constexpr size_t smem_bytes(int bn) { return static_cast<size_t>(kStages) * (kBM * kBK + kBK * bn) * sizeof(bf16); }
+// the stages, and for kSiluGrad the CTA's 128 x 128 tile of pre-activations
+constexpr size_t smem_bytes(int bn, bool silu) {
+    return static_cast<size_t>(kStages) * (kBM * kBK + kBK * bn) * sizeof(bf16) + (silu ? kBM * 128 * sizeof(float) : 0);
+}
+// float offset of the 16-byte chunk (row, c) of the pre-activation tile: the four rows that a half warp of
+// the epilogue reads lie in different banks
+__device__ __forceinline__ int off_z(int row, int c) { return row * 128 + ((c ^ (2 * (row & 3))) << 2); }
 
 __device__ __forceinline__ void cp16(bf16* dst, const bf16* src, int bytes) {
     const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
@@ -379,6 +385,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_bw(const __grid_constant__
         if (s < nk) load_stage<BN, kAM>(g, As + s * kBM * kBK, Bs + s * kBK * BN, m0, n0, k_begin + s * kBK, k_end, tid);
         cp_commit();
     }
+    // kSiluGrad: the pre-activations come with the stages (kSiluGrad is memory-bound: reading them in the epilogue,
+    // with nothing in flight beside them, took as long as the product), the adjoints leave through the same tile
+    float* Zt = reinterpret_cast<float*>(Bs + kStages * kBK * BN);
+    const int zper = kEpi == kSiluGrad ? (16 + nk - 1) / max(nk, 1) : 0;
+    int zi = 0;
     const int mat = lane >> 3, r8 = lane & 7;
     float rs = 0.0f;  // row sums of A: row tid / 2, half tid % 2 of the 32 k of a stage
     for (int kt = 0; kt < nk; ++kt) {
@@ -388,6 +399,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_bw(const __grid_constant__
         if (nt < nk) {
             const int sb = nt % kStages;
             load_stage<BN, kAM>(g, As + sb * kBM * kBK, Bs + sb * kBK * BN, m0, n0, k_begin + nt * kBK, k_end, tid);
+        }
+        if constexpr (kEpi == kSiluGrad) {
+            for (int e = min(16, zi + zper); pairs && zi < e; ++zi) {
+                const int id = tid + zi * kThreads, r = id >> 5, c = id & 31;
+                const int valid = m0 + r < g.M ? max(0, min(4, g.N - n0 - c * 4)) : 0;
+                const float* src = valid > 0 ? g.Zs + static_cast<int64_t>(m0 + r) * g.ldz + n0 + c * 4 : g.Zs;
+                cp16(reinterpret_cast<bf16*>(Zt + off_z(r, c)), reinterpret_cast<const bf16*>(src), 4 * valid);
+            }
         }
         cp_commit();
         const bf16* A_ = As + (kt % kStages) * kBM * kBK;
@@ -435,6 +454,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_bw(const __grid_constant__
         }
     }
     cp_wait<0>();
+    if constexpr (kEpi == kSiluGrad) __syncthreads();  // the pre-activation tile is complete
     if constexpr (kEpi == kAtomic && !kAM) {
         if (g.rowsum != nullptr) {
             rs += __shfl_xor_sync(0xffffffffu, rs, 1);
@@ -474,10 +494,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_bw(const __grid_constant__
                     const float* z = g.Zs + static_cast<int64_t>(row) * g.ldz + col;
                     bf16* q = g.Cb + static_cast<int64_t>(row) * g.ldcb + col;
                     if (two && pairs) {
-                        const float2 zz = *reinterpret_cast<const float2*>(z);
+                        float* zt = Zt + off_z(row - m0, (col - n0) >> 2) + (col & 3);
+                        const float2 zz = *reinterpret_cast<const float2*>(zt);
                         v0 *= silu_grad(zz.x);
                         v1 *= silu_grad(zz.y);
-                        *reinterpret_cast<__nv_bfloat162*>(q) = __floats2bfloat162_rn(v0, v1);
+                        *reinterpret_cast<__nv_bfloat162*>(zt) = __floats2bfloat162_rn(v0, v1);  // over its own z
                     } else {
                         v0 *= silu_grad(z[0]);
                         q[0] = __float2bfloat16(v0);
@@ -493,6 +514,18 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_bw(const __grid_constant__
                 }
             }
     if constexpr (kEpi == kSiluGrad) {
+        if (pairs) {  // eight adjoints (16 bytes) a thread and store
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int id = tid + i * kThreads, r = id >> 4, c8 = id & 15;
+                if (m0 + r >= g.M || n0 + c8 * 8 >= g.N) continue;
+                const uint4 lo = *reinterpret_cast<const uint4*>(Zt + off_z(r, 2 * c8));
+                const uint4 hi = *reinterpret_cast<const uint4*>(Zt + off_z(r, 2 * c8 + 1));
+                *reinterpret_cast<uint4*>(g.Cb + static_cast<int64_t>(m0 + r) * g.ldcb + n0 + c8 * 8) =
+                    make_uint4(lo.x, lo.z, hi.x, hi.z);
+            }
+        }
         if (g.colsum != nullptr) {  // the warp's column sums: over gq (lane bits 2-4), then one atomic
 #pragma unroll
             for (int j = 0; j < NJ; ++j)
@@ -838,66 +871,70 @@ __global__ void k_spline_inverse(int64_t B, int d, int K, const float* Xin, floa
 // of x^(l+1) in gXn (the conditioning dims get the MLP part later).
 template <int kK>
 __global__ void k_spline_backward(int64_t B, int d, int K, const float* Xl, const float* Praw, int64_t ldp,
-                                  const __grid_constant__ LayerDesc ld, const float* gX, const double* wtot,
-                                  const double* wsum, float* G, bf16* Gb, float* gXn, double* loss) {
-    int64_t b = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-    float lsum = 0.0f;
-    if (b < B) {
-        const float c = wsum[0] > 0.0 ? static_cast<float>(wtot[b] / wsum[0]) : 0.0f;
-        for (int j = 0; j < d; ++j) gXn[b * d + j] = gX[b * d + j];  // A dims pass through
-        const float cw = 1.0f - K * kMinW, chh = 1.0f - K * kMinH;
-        for (int q = 0; q < ld.nb; ++q) {
-            const int64_t row0 = static_cast<int64_t>(q) * (3 * K + 1);
-            const float* raw = Praw + row0 * ldp + b;
-            int j = ld.tb[q];
-            float xv = fminf(fmaxf(Xl[b * d + j], 0.0f), 1.0f);
-            Bin bn = locate_k<kK>(raw, ldp, K, xv, false);
-            Dual F, Fp;
-            bin_eval<Dual>(dvar(xv, 0), dvar(bn.x0, 1), dvar(bn.w, 2), dvar(bn.y0, 3), dvar(bn.h, 4), dvar(bn.d0, 5),
-                           dvar(bn.d1, 6), F, Fp);
-            float ifp = 1.0f / Fp.v;
-            lsum += c * logf(Fp.v);
-            float ax = gX[b * d + j] + c * Fp.t[0] * ifp;  // adjoint of x^(l)_j incl. d(c log F')/dx
-            gXn[b * d + j] = ax * ifp;                       // d x^(l) / d x^(l+1) = 1/F'
-            // bin-parameter adjoints: -a_x F_theta / F' + c F'_theta / F'
-            float gt[7];
-#pragma unroll
-            for (int i = 1; i < 7; ++i) gt[i] = (-ax * F.t[i] + c * Fp.t[i]) * ifp;
-            // chain to the raw parameters: x_k = sum_{i<k} w_i and w_k through the width softmax,
-            // y_k and h_k through the height softmax, d_k and d_{k+1} through softplus
-            const float dotw = gt[1] * bn.sx + gt[2] * bn.pw;
-            const float doth = gt[3] * bn.sy + gt[4] * bn.ph;
-            float* g = G ? G + row0 * ldp + b : nullptr;
-            bf16* gb = Gb + row0 * ldp + b;
-            const float nmw = -bn.mw * kLog2e, nmh = -bn.mh * kLog2e;
-            for (int i = 0; i < K; ++i) {
-                float pw = softmax_exp(raw[i * ldp], nmw) * bn.iw;
-                float ph = softmax_exp(raw[(K + i) * ldp], nmh) * bn.ih;
-                float aw = i < bn.k ? gt[1] : (i == bn.k ? gt[2] : 0.0f);
-                float ah = i < bn.k ? gt[3] : (i == bn.k ? gt[4] : 0.0f);
-                float vw = cw * pw * (aw - dotw), vh = chh * ph * (ah - doth);
-                if (G) {
-                    g[i * ldp] = vw;
-                    g[(K + i) * ldp] = vh;
-                }
-                gb[i * ldp] = __float2bfloat16(vw);
-                gb[(K + i) * ldp] = __float2bfloat16(vh);
-            }
-            for (int i = 0; i <= K; ++i) {
-                float v = i == bn.k ? gt[5] * bn.sg0 : (i == bn.k + 1 ? gt[6] * bn.sg1 : 0.0f);
-                if (G) g[(2 * K + i) * ldp] = v;
-                gb[(2 * K + i) * ldp] = __float2bfloat16(v);
-            }
-        }
+                                  const __grid_constant__ LayerDesc ld, const float* gX, const float* cw_ev,
+                                  float* G, bf16* Gb, float* gXn, float* lterm) {
+    const int64_t b = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (b >= B) return;
+    const int q = blockIdx.y;
+    if (q == 0) {
+        for (int i = 0; i < ld.na; ++i) gXn[b * d + ld.ta[i]] = gX[b * d + ld.ta[i]];  // A dims pass through
         for (int p = ld.P; p < ld.Ppad; ++p) {
             if (G) G[p * ldp + b] = 0.0f;
             Gb[p * ldp + b] = __float2bfloat16(0.0f);
         }
     }
-    // loss = sum_b c_b sum log F'  (one atomic per warp)
+    const float c = cw_ev[b];
+    const float cw = 1.0f - K * kMinW, chh = 1.0f - K * kMinH;
+    const int64_t row0 = static_cast<int64_t>(q) * (3 * K + 1);
+    const float* raw = Praw + row0 * ldp + b;
+    const int j = ld.tb[q];
+    const float xv = fminf(fmaxf(Xl[b * d + j], 0.0f), 1.0f);
+    Bin bn = locate_k<kK>(raw, ldp, K, xv, false);
+    Dual F, Fp;
+    bin_eval<Dual>(dvar(xv, 0), dvar(bn.x0, 1), dvar(bn.w, 2), dvar(bn.y0, 3), dvar(bn.h, 4), dvar(bn.d0, 5),
+                   dvar(bn.d1, 6), F, Fp);
+    float ifp = 1.0f / Fp.v;
+    lterm[q * ldp + b] = logf(Fp.v);
+    float ax = gX[b * d + j] + c * Fp.t[0] * ifp;  // adjoint of x^(l)_j incl. d(c log F')/dx
+    gXn[b * d + j] = ax * ifp;                       // d x^(l) / d x^(l+1) = 1/F'
+    // bin-parameter adjoints: -a_x F_theta / F' + c F'_theta / F'
+    float gt[7];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, static_cast<double>(lsum));
+    for (int i = 1; i < 7; ++i) gt[i] = (-ax * F.t[i] + c * Fp.t[i]) * ifp;
+    // chain to the raw parameters: x_k = sum_{i<k} w_i and w_k through the width softmax,
+    // y_k and h_k through the height softmax, d_k and d_{k+1} through softplus
+    const float dotw = gt[1] * bn.sx + gt[2] * bn.pw;
+    const float doth = gt[3] * bn.sy + gt[4] * bn.ph;
+    float* g = G ? G + row0 * ldp + b : nullptr;
+    bf16* gb = Gb + row0 * ldp + b;
+    const float nmw = -bn.mw * kLog2e, nmh = -bn.mh * kLog2e;
+    const int Kc = kK > 0 ? kK : K;
+#pragma unroll
+    for (int i = 0; i < Kc; ++i) {
+        float pw = softmax_exp(raw[i * ldp], nmw) * bn.iw;
+        float ph = softmax_exp(raw[(Kc + i) * ldp], nmh) * bn.ih;
+        float aw = i < bn.k ? gt[1] : (i == bn.k ? gt[2] : 0.0f);
+        float ah = i < bn.k ? gt[3] : (i == bn.k ? gt[4] : 0.0f);
+        float vw = cw * pw * (aw - dotw), vh = chh * ph * (ah - doth);
+        if (G) {
+            g[i * ldp] = vw;
+            g[(Kc + i) * ldp] = vh;
+        }
+        gb[i * ldp] = __float2bfloat16(vw);
+        gb[(Kc + i) * ldp] = __float2bfloat16(vh);
+    }
+#pragma unroll
+    for (int i = 0; i <= Kc; ++i) {
+        float v = i == bn.k ? gt[5] * bn.sg0 : (i == bn.k + 1 ? gt[6] * bn.sg1 : 0.0f);
+        if (G) g[(2 * Kc + i) * ldp] = v;
+        gb[(2 * Kc + i) * ldp] = __float2bfloat16(v);
+    }
+}
+
+// c_b = w_b / sum w, the events' weights in the loss (once per backward pass: the FP64 quotient is not the layers' work)
+__global__ void k_event_weight(int64_t B, const double* wtot, const double* wsum, float* cw) {
+    const int64_t b = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (b < B) cw[b] = wsum[0] > 0.0 ? static_cast<float>(wtot[b] / wsum[0]) : 0.0f;
 }
 
 // row sums of an [n][ldm] fp32 matrix over its first B columns into out[n] (atomic; bias
@@ -931,10 +968,20 @@ __global__ void k_colsum(int64_t B, int n, const float* M, float* out) {
     atomicAdd(out + col, s);
 }
 
-__global__ void k_scatter(int64_t B, int d, const __grid_constant__ LayerDesc ld, const float* dIn, float* gXn) {
+// adds the adjoints of the conditioning dims and the layer's part of the loss, sum_b c_b sum_q log F' (the terms of
+// an event in order, one atomic per warp)
+__global__ void k_scatter(int64_t B, int d, const __grid_constant__ LayerDesc ld, const float* dIn, float* gXn,
+                          const float* cw, const float* lterm, int64_t ldp, double* loss) {
     int64_t b = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-    if (b >= B) return;
-    for (int i = 0; i < ld.na; ++i) gXn[b * d + ld.ta[i]] += dIn[b * kInPad + i];
+    float lsum = 0.0f;
+    if (b < B) {
+        for (int i = 0; i < ld.na; ++i) gXn[b * d + ld.ta[i]] += dIn[b * kInPad + i];
+        const float c = cw[b];
+        for (int q = 0; q < ld.nb; ++q) lsum = fmaf(c, lterm[q * ldp + b], lsum);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(loss, static_cast<double>(lsum));
 }
 
 // w_b = w_map_b exp(logdet_b) (the flow density is 1/|dr/dz|); block sums into wsum
@@ -1823,6 +1870,8 @@ struct ps_flow_s {
     float* gX = nullptr;     // [max_batch][d]
     float* gXn = nullptr;
     double* wtot = nullptr;  // [max_batch]
+    float* cw = nullptr;     // [max_batch] w / sum w
+    float* lterm = nullptr;  // [transformed dims of a layer][max_batch] log F'
     double* scal = nullptr;  // [0] sum w, [1] loss
     int Pmax = 0;
     // buffers of the fused sampling / density path (allocated on first use)
@@ -1844,7 +1893,7 @@ void free_flow(ps_flow f) {
                     static_cast<void*>(f->logdet), static_cast<void*>(f->G), static_cast<void*>(f->Gb),
                     static_cast<void*>(f->dA), static_cast<void*>(f->dZ), static_cast<void*>(f->dZb), static_cast<void*>(f->dAb),
                     static_cast<void*>(f->dIn), static_cast<void*>(f->gX), static_cast<void*>(f->gXn),
-                    static_cast<void*>(f->wtot), static_cast<void*>(f->scal),
+                    static_cast<void*>(f->wtot), static_cast<void*>(f->cw), static_cast<void*>(f->lterm), static_cast<void*>(f->scal),
                     static_cast<void*>(f->gen_X), static_cast<void*>(f->gen_ld),
                     static_cast<void*>(f->gen_status)})
         cudaFree(q);
@@ -1889,8 +1938,9 @@ bool gemm_bw(bwg::Args a, bool am, int epi, int splits, cudaStream_t st, int* st
     const dim3 grid((a.M + bwg::kBM - 1) / bwg::kBM, (a.N + bn - 1) / bn, nz);
     int pairs = 0;
     if (epi == bwg::kStore) pairs = al(a.C, 7) && a.ldc % 2 == 0;
-    if (epi == bwg::kSiluGrad) pairs = al(a.Zs, 7) && a.ldz % 2 == 0 && al(a.Cb, 3) && a.ldcb % 2 == 0;
-    const size_t smem = bwg::smem_bytes(bn);
+    // kSiluGrad: 16-byte copies of the pre-activations and stores of the adjoints
+    if (epi == bwg::kSiluGrad) pairs = al(a.Zs, 15) && a.ldz % 4 == 0 && al(a.Cb, 15) && a.ldcb % 8 == 0 && a.N % 8 == 0;
+    const size_t smem = bwg::smem_bytes(bn, epi == bwg::kSiluGrad);
     const int key = (narrow ? 100 : 0) + (am ? 10 : 0) + epi;
     switch (key) {
         case 0 + bwg::kAtomic: bwg::k_gemm_bw<128, false, bwg::kAtomic><<<grid, bwg::kThreads, smem, st>>>(a, pairs); break;
@@ -2014,13 +2064,16 @@ int inverse(ps_flow f, int64_t B, cudaStream_t st) {
     return fcheck(cudaGetLastError(), "flow inverse");
 }
 
+constexpr int kSplineThreads = 128;  // events per block of k_spline_backward (one transformed dim per block row)
+
 // backward sweep (layers 0 .. L-1) of the importance-weighted forward KL; accumulates f->grad
 int backward(ps_flow f, int64_t B, cudaStream_t st) {
     const FlowDesc& fd = f->fd;
     const int d = fd.d, H = fd.H, T = 256;
     cudaMemsetAsync(f->gX, 0, B * d * sizeof(float), st);
     cudaMemsetAsync(f->grad, 0, f->n_params * sizeof(float), st);
-    int launches = 0;
+    int launches = 1;
+    k_event_weight<<<blocks(B, T), T, 0, st>>>(B, f->wtot, f->scal, f->cw);
     const unsigned colsum_rows = static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(512, B / 64)));
     // batch-long weight-gradient GEMMs: split the batch so that about two CTAs per SM run,
     // with at least 256 events per split
@@ -2054,8 +2107,9 @@ int backward(ps_flow f, int64_t B, cudaStream_t st) {
         w.M = ld.Ppad; w.N = H; w.K = Bi; w.C = f->grad + ld.off_W3; w.ldc = H; w.rowsum = f->grad + ld.off_b3;
         const bool fast3 = gemm_bw_fits(w, false);
         auto kb = fd.K == 16 ? k_spline_backward<16> : k_spline_backward<0>;
-        kb<<<blocks(B, T), T, 0, st>>>(B, d, fd.K, Xl, P, ldg, ld, f->gX, f->wtot, f->scal, fast3 ? nullptr : f->G,
-                                       f->Gb, f->gXn, f->scal + 1);
+        kb<<<dim3(blocks(B, kSplineThreads), ld.nb), kSplineThreads, 0, st>>>(B, d, fd.K, Xl, P, ldg, ld, f->gX, f->cw,
+                                                                             fast3 ? nullptr : f->G, f->Gb, f->gXn,
+                                                                             f->lterm);
         if (!fast3 || !gemm_bw(w, false, bwg::kAtomic, split_bw(ld.Ppad, H), st, &s)) {
             k_rowsum<<<dim3(std::min<unsigned>(blocks(B, 256), 4), ld.Ppad), 256, 0, st>>>(B, ldg, f->G,
                                                                                              f->grad + ld.off_b3);
@@ -2131,7 +2185,7 @@ int backward(ps_flow f, int64_t B, cudaStream_t st) {
             s = gemm(g, 1, st);
         }
         if (s != PS_OK) return s;
-        k_scatter<<<blocks(B, T), T, 0, st>>>(B, d, ld, f->dIn, f->gXn);
+        k_scatter<<<blocks(B, T), T, 0, st>>>(B, d, ld, f->dIn, f->gXn, f->cw, f->lterm, ldg, f->scal + 1);
         std::swap(f->gX, f->gXn);
         launches += 2;  // spline backward, scatter (the GEMMs count themselves)
     }
@@ -2319,6 +2373,11 @@ int ps_flow_create(int dims, int n_layers, int bins, int hidden, int64_t max_bat
     auto alloc = [&](void** q, size_t bytes) {
         if (st == PS_OK) st = fcheck(cudaMalloc(q, std::max<size_t>(bytes, 256)), "cudaMalloc (flow)");
     };
+    for (auto kern : {bwg::k_gemm_bw<128, false, bwg::kSiluGrad>, bwg::k_gemm_bw<128, true, bwg::kSiluGrad>})
+        if (st == PS_OK)
+            st = fcheck(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             static_cast<int>(bwg::smem_bytes(128, true))),
+                        "cudaFuncSetAttribute");
     const int64_t B = max_batch, H = hidden, L = n_layers;
     alloc(reinterpret_cast<void**>(&f->p), off * 4);
     alloc(reinterpret_cast<void**>(&f->grad), off * 4);
@@ -2343,6 +2402,8 @@ int ps_flow_create(int dims, int n_layers, int bins, int hidden, int64_t max_bat
     alloc(reinterpret_cast<void**>(&f->gX), B * dims * 4);
     alloc(reinterpret_cast<void**>(&f->gXn), B * dims * 4);
     alloc(reinterpret_cast<void**>(&f->wtot), B * 8);
+    alloc(reinterpret_cast<void**>(&f->cw), B * 4);
+    alloc(reinterpret_cast<void**>(&f->lterm), B * dims * 4);
     alloc(reinterpret_cast<void**>(&f->scal), 2 * 8);
     if (st == PS_OK) st = fcheck(cudaMemcpy(f->p, h.data(), off * 4, cudaMemcpyHostToDevice), "upload flow params");
     if (st == PS_OK) st = fcheck(cudaMemset(f->m, 0, off * 4), "memset");

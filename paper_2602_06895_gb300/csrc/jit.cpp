@@ -164,14 +164,16 @@ std::string channel_weight_source(const Compiled& C, const int32_t* a, int na, b
             var = it->second;
         } else {
             var = "cw" + std::to_string(memo->next++);
-            std::string q = kind == 1 ? ldp + std::to_string(a[1]) + ")"
-                                      : (mixed ? "dev::mx::F4{0.0f, 0.0f, 0.0f, 0.0f}" : "dev::P4{0.0, 0.0, 0.0, 0.0}");
+            // a sum starts from its first momentum: 0 + x does not fold (x = -0), and the square has no sign
+            std::string q = kind == 1 ? ldp + std::to_string(a[1]) + ")" : std::string();
             for (int i = 0; i < k; ++i) {
                 if (!((mask >> i) & 1)) continue;
+                const std::string p = ldp + std::to_string(a[2 + i]) + ")";
                 const std::string fn = mixed ? (kind == 1 ? "dev::mx::f4_sub(" : "dev::mx::f4_add(")
                                              : (kind == 1 ? "dev::p4_sub(" : "dev::p4_add(");
-                q = fn + q + ", " + ldp + std::to_string(a[2 + i]) + "))";
+                q = q.empty() ? p : fn + q + ", " + p + ")";
             }
+            if (q.empty()) q = mixed ? "dev::mx::F4{0.0f, 0.0f, 0.0f, 0.0f}" : "dev::P4{0.0, 0.0, 0.0, 0.0}";
             *decl += mixed ? "                const float " + var + " = dev::mx::sde_sq(" + q + ");\n"
                            : "                const double " + var + " = dev::p4_sq(" + q + ");\n";
             memo->names[form] = var;
@@ -462,11 +464,11 @@ Plan make_plan(const std::vector<Compiled>& ch, int block, int min_blocks, bool 
         p.max_regs = register_cap(block, min_blocks);
         // Without a request, an FP64 channel whose slot file (two registers a slot) leaves room for the
         // arithmetic in 168 registers is held to them: 12 warps an SM instead of 8 hide the FP64 latency
-        // (2->5, 60 slots, 4e6 events: 6.5 against 6.9 ms); a larger one would spill (2->8, 85 slots: 5.20
+        // (2->5, 62 slots, 4e6 events: 6.5 against 6.7 ms); a larger one would spill (2->8, 85 slots: 5.20
         // against 4.91 ms per 2^20).
         int slots = 0;
         for (const Compiled& c : ch) slots = std::max(slots, c.n_slots);
-        if (!mixed && min_blocks <= 0 && slots <= 60) p.max_regs = register_cap(128, 3);
+        if (!mixed && min_blocks <= 0 && slots <= 64) p.max_regs = register_cap(128, 3);
         p.units = jit_sources_split(ch, block, min_blocks, mixed);
         for (const std::string& u : p.units) p.key += u + "\n// ---- unit\n";
         p.key += "// maxrregcount " + std::to_string(p.max_regs) + "\n";
