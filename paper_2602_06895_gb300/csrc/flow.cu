@@ -2105,7 +2105,7 @@ int backward(ps_flow f, int64_t B, cudaStream_t st) {
         bwg::Args w{};
         w.A = f->Gb; w.lam = ldg; w.lak = 1; w.B = A2; w.ldb = H;
         w.M = ld.Ppad; w.N = H; w.K = Bi; w.C = f->grad + ld.off_W3; w.ldc = H; w.rowsum = f->grad + ld.off_b3;
-        const bool fast3 = gemm_bw_fits(w, false);
+        const bool fast3 = H > 16 && gemm_bw_fits(w, false);  // k_gemm takes the products 16 columns wide
         auto kb = fd.K == 16 ? k_spline_backward<16> : k_spline_backward<0>;
         kb<<<dim3(blocks(B, kSplineThreads), ld.nb), kSplineThreads, 0, st>>>(B, d, fd.K, Xl, P, ldg, ld, f->gX, f->cw,
                                                                              fast3 ? nullptr : f->G, f->Gb, f->gXn,
