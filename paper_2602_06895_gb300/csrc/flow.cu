@@ -279,7 +279,7 @@ struct Args {
     int64_t ldz;
     bf16* Cb;          // kSiluGrad: the adjoint as bfloat16, Cb[m * ldcb + n]
     int64_t ldcb;
-    float* colsum;     // kSiluGrad: column sums of the adjoint (bias gradient), atomic
+    float* colsum;     // kSiluGrad: column sums of the adjoint over each CTA's rows, colsum[blockIdx.x * N + n]
     float* rowsum;     // kAtomic with A unit-stride along k: row sums of A (bias gradient), atomic
 };
 
@@ -526,7 +526,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_bw(const __grid_constant__
                     make_uint4(lo.x, lo.z, hi.x, hi.z);
             }
         }
-        if (g.colsum != nullptr) {  // the warp's column sums: over gq (lane bits 2-4), then one atomic
+        // The CTA's column sums, over gq (lane bits 2-4) and the two warp rows, as one row of partials that k_scatter
+        // adds up.  One atomic a warp and column put 131072 adds on 128 addresses: at 65536 events and width 128 the
+        // two products of a layer took 40.4 and 34.0 us with them and take 35.6 and 27.8 us without.
+        float* S = reinterpret_cast<float*>(As);  // the stages are read no more
+        if (g.colsum != nullptr) {
 #pragma unroll
             for (int j = 0; j < NJ; ++j)
 #pragma unroll
@@ -535,9 +539,15 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_bw(const __grid_constant__
                     s += __shfl_xor_sync(0xffffffffu, s, 4);
                     s += __shfl_xor_sync(0xffffffffu, s, 8);
                     s += __shfl_xor_sync(0xffffffffu, s, 16);
-                    const int col = n0 + wn0 + j * 8 + 2 * tq + e;
-                    if (gq == 0 && col < g.N && m0 + wm0 < g.M) atomicAdd(g.colsum + col, s);
+                    if (gq == 0) S[(warp / WN) * BN + wn0 + j * 8 + 2 * tq + e] = s;
                 }
+            __syncthreads();
+            if (tid < BN && n0 + tid < g.N) {
+                float s = 0.0f;
+#pragma unroll
+                for (int r = 0; r < WM; ++r) s += S[r * BN + tid];
+                g.colsum[static_cast<int64_t>(blockIdx.x) * g.N + n0 + tid] = s;
+            }
         }
     }
 }
@@ -968,11 +978,46 @@ __global__ void k_colsum(int64_t B, int n, const float* M, float* out) {
     atomicAdd(out + col, s);
 }
 
+// Column sums of the adjoints of a layer's two hidden biases, from the partial rows of their GEMMs
+struct BiasSums {
+    const float* part[2];  // [rows][n]
+    float* out[2];         // nullptr: summed elsewhere
+    int rows, n;
+};
+constexpr int kScatterThreads = 256;
+
 // adds the adjoints of the conditioning dims and the layer's part of the loss, sum_b c_b sum_q log F' (the terms of
-// an event in order, one atomic per warp)
-__global__ void k_scatter(int64_t B, int d, const __grid_constant__ LayerDesc ld, const float* dIn, float* gXn,
-                          const float* cw, const float* lterm, int64_t ldp, double* loss) {
-    int64_t b = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+// an event in order, one atomic per warp).  The first blocks take the column sums of the layer's hidden biases beside
+// that: eight columns (one sector) a block and 32 threads a column, in an order that does not depend on the schedule
+__global__ void __launch_bounds__(kScatterThreads) k_scatter(int64_t B, int d, const __grid_constant__ LayerDesc ld,
+                                                             const float* dIn, float* gXn, const float* cw,
+                                                             const float* lterm, int64_t ldp, double* loss,
+                                                             const __grid_constant__ BiasSums bs) {
+    __shared__ float s_part[kScatterThreads / 4];
+    const int groups = (bs.n + 7) / 8;
+    if (static_cast<int>(blockIdx.x) < 2 * groups) {
+        const int which = static_cast<int>(blockIdx.x) >= groups;
+        const int col = 8 * (static_cast<int>(blockIdx.x) - which * groups) + (threadIdx.x & 7);
+        if (bs.out[which] == nullptr) return;
+        float s = 0.0f;
+        if (col < bs.n) {
+#pragma unroll 16
+            for (int r = threadIdx.x >> 3; r < bs.rows; r += kScatterThreads / 8)
+                s += bs.part[which][static_cast<int64_t>(r) * bs.n + col];
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 8);
+        s += __shfl_xor_sync(0xffffffffu, s, 16);
+        if ((threadIdx.x & 31) < 8) s_part[(threadIdx.x >> 5) * 8 + (threadIdx.x & 7)] = s;
+        __syncthreads();
+        if (threadIdx.x < 8 && col < bs.n) {
+            s = 0.0f;
+#pragma unroll
+            for (int w = 0; w < kScatterThreads / 32; ++w) s += s_part[w * 8 + threadIdx.x];
+            bs.out[which][col] = s;
+        }
+        return;
+    }
+    int64_t b = (blockIdx.x - 2 * groups) * static_cast<int64_t>(blockDim.x) + threadIdx.x;
     float lsum = 0.0f;
     if (b < B) {
         for (int i = 0; i < ld.na; ++i) gXn[b * d + ld.ta[i]] += dIn[b * kInPad + i];
@@ -1872,6 +1917,7 @@ struct ps_flow_s {
     double* wtot = nullptr;  // [max_batch]
     float* cw = nullptr;     // [max_batch] w / sum w
     float* lterm = nullptr;  // [transformed dims of a layer][max_batch] log F'
+    float* colpart = nullptr;  // [2][max_batch / 128][H] column sums of the hidden adjoints, one row a CTA
     double* scal = nullptr;  // [0] sum w, [1] loss
     int Pmax = 0;
     // buffers of the fused sampling / density path (allocated on first use)
@@ -1893,7 +1939,7 @@ void free_flow(ps_flow f) {
                     static_cast<void*>(f->logdet), static_cast<void*>(f->G), static_cast<void*>(f->Gb),
                     static_cast<void*>(f->dA), static_cast<void*>(f->dZ), static_cast<void*>(f->dZb), static_cast<void*>(f->dAb),
                     static_cast<void*>(f->dIn), static_cast<void*>(f->gX), static_cast<void*>(f->gXn),
-                    static_cast<void*>(f->wtot), static_cast<void*>(f->cw), static_cast<void*>(f->lterm), static_cast<void*>(f->scal),
+                    static_cast<void*>(f->wtot), static_cast<void*>(f->cw), static_cast<void*>(f->lterm), static_cast<void*>(f->colpart), static_cast<void*>(f->scal),
                     static_cast<void*>(f->gen_X), static_cast<void*>(f->gen_ld),
                     static_cast<void*>(f->gen_status)})
         cudaFree(q);
@@ -2074,6 +2120,7 @@ int backward(ps_flow f, int64_t B, cudaStream_t st) {
     cudaMemsetAsync(f->grad, 0, f->n_params * sizeof(float), st);
     int launches = 1;
     k_event_weight<<<blocks(B, T), T, 0, st>>>(B, f->wtot, f->scal, f->cw);
+    const int64_t part_rows = (f->max_batch + bwg::kBM - 1) / bwg::kBM;  // rows of a bias gradient's partials
     const unsigned colsum_rows = static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(512, B / 64)));
     // batch-long weight-gradient GEMMs: split the batch so that about two CTAs per SM run,
     // with at least 256 events per split
@@ -2124,7 +2171,10 @@ int backward(ps_flow f, int64_t B, cudaStream_t st) {
         w = bwg::Args{};
         w.A = f->Gb; w.lam = 1; w.lak = ldg; w.B = f->pb + ld.off_W3; w.ldb = H;
         w.M = Bi; w.N = H; w.K = ld.Ppad; w.Zs = Z2; w.ldz = H; w.Cb = f->dZb; w.ldcb = H;
-        w.colsum = f->grad + ld.off_b2;
+        w.colsum = f->colpart;
+        BiasSums bs{{f->colpart, f->colpart + part_rows * H},
+                    {f->grad + ld.off_b2, f->grad + ld.off_b1},
+                    static_cast<int>((B + bwg::kBM - 1) / bwg::kBM), H};
         if (!gemm_bw(w, true, bwg::kSiluGrad, 1, st, &s)) {
             GemmArgs g{};
             g.A = f->Gb; g.lam = 1; g.lak = ldg; g.B = f->pb + ld.off_W3; g.lbn = 1; g.lbk = H;
@@ -2133,6 +2183,7 @@ int backward(ps_flow f, int64_t B, cudaStream_t st) {
             s = gemm(g, 1, st);
             if (s == PS_OK) {
                 k_colsum<<<dim3(blocks(H, 64), colsum_rows), 64, 0, st>>>(B, H, f->dZ, f->grad + ld.off_b2);
+                bs.out[0] = nullptr;
                 launches += 1;
             }
         }
@@ -2151,7 +2202,7 @@ int backward(ps_flow f, int64_t B, cudaStream_t st) {
         w = bwg::Args{};
         w.A = f->dZb; w.lam = H; w.lak = 1; w.B = f->pb + ld.off_W2; w.ldb = H;
         w.M = Bi; w.N = H; w.K = H; w.Zs = Z1; w.ldz = H; w.Cb = f->dAb; w.ldcb = H;
-        w.colsum = f->grad + ld.off_b1;
+        w.colsum = f->colpart + part_rows * H;
         if (!gemm_bw(w, false, bwg::kSiluGrad, 1, st, &s)) {
             GemmArgs g{};
             g.A = f->dZb; g.lam = H; g.lak = 1; g.B = f->pb + ld.off_W2; g.lbn = 1; g.lbk = H;
@@ -2160,6 +2211,7 @@ int backward(ps_flow f, int64_t B, cudaStream_t st) {
             s = gemm(g, 1, st);
             if (s == PS_OK) {
                 k_colsum<<<dim3(blocks(H, 64), colsum_rows), 64, 0, st>>>(B, H, f->dA, f->grad + ld.off_b1);
+                bs.out[1] = nullptr;
                 launches += 1;
             }
         }
@@ -2185,7 +2237,8 @@ int backward(ps_flow f, int64_t B, cudaStream_t st) {
             s = gemm(g, 1, st);
         }
         if (s != PS_OK) return s;
-        k_scatter<<<blocks(B, T), T, 0, st>>>(B, d, ld, f->dIn, f->gXn, f->cw, f->lterm, ldg, f->scal + 1);
+        k_scatter<<<2 * ((H + 7) / 8) + blocks(B, kScatterThreads), kScatterThreads, 0, st>>>(
+            B, d, ld, f->dIn, f->gXn, f->cw, f->lterm, ldg, f->scal + 1, bs);
         std::swap(f->gX, f->gXn);
         launches += 2;  // spline backward, scatter (the GEMMs count themselves)
     }
@@ -2404,6 +2457,7 @@ int ps_flow_create(int dims, int n_layers, int bins, int hidden, int64_t max_bat
     alloc(reinterpret_cast<void**>(&f->wtot), B * 8);
     alloc(reinterpret_cast<void**>(&f->cw), B * 4);
     alloc(reinterpret_cast<void**>(&f->lterm), B * dims * 4);
+    alloc(reinterpret_cast<void**>(&f->colpart), 2 * ((B + bwg::kBM - 1) / bwg::kBM) * hidden * 4);
     alloc(reinterpret_cast<void**>(&f->scal), 2 * 8);
     if (st == PS_OK) st = fcheck(cudaMemcpy(f->p, h.data(), off * 4, cudaMemcpyHostToDevice), "upload flow params");
     if (st == PS_OK) st = fcheck(cudaMemset(f->m, 0, off * 4), "memset");

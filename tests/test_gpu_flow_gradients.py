@@ -16,7 +16,7 @@ from test_gpu_flow import random_params, sample, torch_cuda  # noqa: F401
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("hidden,B", [(16, 130), (48, 257)])
+@pytest.mark.parametrize("hidden,B", [(128, 1), (128, 127), (128, 129), (16, 130), (48, 257), (144, 1025)])
 def test_last_events_gradients(torch_cuda, hidden, B):  # noqa: F811
     torch = torch_cuda
     fl = ps.Flow(5, 4, 8, hidden, max_batch=2048)
