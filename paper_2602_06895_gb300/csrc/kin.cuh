@@ -108,48 +108,12 @@ __device__ __forceinline__ P4 p4_add(P4 a, P4 b) { return {a.e + b.e, a.x + b.x,
 __device__ __forceinline__ P4 p4_sub(P4 a, P4 b) { return {a.e - b.e, a.x - b.x, a.y - b.y, a.z - b.z}; }
 __device__ __forceinline__ double p4_sq(P4 a) { return a.e * a.e - a.x * a.x - a.y * a.y - a.z * a.z; }
 
-// Kallen lambda(x, y, z) = (x - y - z)^2 - 4 y z (x >= 0), without cancellation:
-//   y, z >= 0: (x - (sqrt y + sqrt z)^2)(x - (sqrt y - sqrt z)^2)
-//   y, z <= 0: x^2 + 2x(|y| + |z|) + (|y| - |z|)^2  (space-like legs of a t-chain)
-//   mixed:     (x - y - z)^2 - 4 y z                (-4yz >= 0)
-// clamped at zero.
-// The branches are taken on the bit patterns (integer ALU); y = z = 0 (two massless legs) is x^2.
 __device__ __forceinline__ bool zero_bits(double v) { return (dbits(v) << 1) == 0; }       // +-0
 __device__ __forceinline__ bool nonneg_bits(double v) { return dbits(v) >= 0 || zero_bits(v); }
 __device__ __forceinline__ bool nonpos_bits(double v) { return dbits(v) <= 0; }            // includes -0
-__device__ __forceinline__ double kallen(double x, double y, double z) {
-    double l;
-    if (zero_bits(y) && zero_bits(z)) {
-        l = x * x;
-    } else if (nonneg_bits(y) && nonneg_bits(z)) {
-        double ry = sqrt(y), rz = sqrt(z);
-        double hi = ry + rz, lo = ry - rz;
-        l = (x - hi * hi) * (x - lo * lo);
-    } else if (nonpos_bits(y) && nonpos_bits(z)) {
-        double d = z - y;
-        l = x * x - 2.0 * x * (y + z) + d * d;
-    } else {
-        double d = x - y - z;
-        l = d * d - 4.0 * y * z;
-    }
-    return pos_bits(l) ? l : 0.0;  // clamped at zero (NaN -> 0)
-}
-// lambda(x, m1^2, m2^2) from the masses m1, m2 >= 0 themselves: the factorised form above with
-// sqrt(m^2) replaced by m.  For a double m the correctly rounded sqrt of fl(m^2) is m exactly
-// (its error is below half an ulp of m), so this equals kallen(x, m1 m1, m2 m2) bit for bit,
-// without the two square roots.
-__device__ __forceinline__ double kallen_m(double x, double m1, double m2) {
-    double l;
-    if (zero_bits(m1 * m1) && zero_bits(m2 * m2)) {
-        l = x * x;
-    } else {
-        double hi = m1 + m2, lo = m1 - m2;
-        l = fma(-hi, hi, x) * fma(-lo, lo, x);  // explicit: the same roundings with constant masses
-    }
-    return pos_bits(l) ? l : 0.0;
-}
-// kallen_m for the forward kernels (masses compared with zero on their words), and its root: x itself for
-// two massless legs
+// lambda(x, m1^2, m2^2) from the masses m1, m2 >= 0 themselves: the factorised form of kallen_in with
+// sqrt(m^2) replaced by m.  For a double m the correctly rounded sqrt of fl(m^2) is m exactly (its
+// error is below half an ulp of m), so no square root is taken.  Its root: x itself for two massless legs.
 __device__ __forceinline__ double kallen_out(double x, double m1, double m2) {
     double l;
     if (is_zero(m1) && is_zero(m2)) {
@@ -175,11 +139,6 @@ struct BoostFrame {
 __device__ __forceinline__ BoostFrame boost_frame(const P4& q, double mq, double inv_m) {
     return {q.e, q.x, q.y, q.z, inv_m, fast::rcp(mq * (q.e + mq))};
 }
-__device__ __forceinline__ P4 boost_out(const P4& p, const BoostFrame& b) {
-    double qp = b.x * p.x + b.y * p.y + b.z * p.z;
-    double c = fma(qp, b.k, p.e * b.inv_m);
-    return {(b.e * p.e + qp) * b.inv_m, p.x + b.x * c, p.y + b.y * c, p.z + b.z * c};
-}
 // The back-to-back daughters q1 = (e1, v) and q2 = (e2, -v) of a two-body decay, boosted out of
 // the same frame: q2 . b = -(q1 . b) exactly, so the dot product is formed once.
 __device__ __forceinline__ void boost_out_pair(const P4& q1, double e2, const BoostFrame& b, P4& p1, P4& p2) {
@@ -194,47 +153,19 @@ __device__ __forceinline__ P4 boost_in(const P4& p, const BoostFrame& b) {
     return {(b.e * p.e - qp) * b.inv_m, p.x + b.x * c, p.y + b.y * c, p.z + b.z * c};
 }
 
-// Pure boost of p from the rest frame of q (invariant mass mq) to the frame where q is given.
-__device__ __forceinline__ P4 boost_out(P4 p, P4 q, double mq) {
-    double qp = q.x * p.x + q.y * p.y + q.z * p.z;
-    double inv = 1.0 / mq;
-    double c = qp / (mq * (q.e + mq)) + p.e * inv;
-    return {(q.e * p.e + qp) * inv, p.x + q.x * c, p.y + q.y * c, p.z + q.z * c};
-}
-
-// The inverse boost: p given in the frame of q -> rest frame of q.
-__device__ __forceinline__ P4 boost_in(P4 p, P4 q, double mq) {
-    double qp = q.x * p.x + q.y * p.y + q.z * p.z;
-    double inv = 1.0 / mq;
-    double c = qp / (mq * (q.e + mq)) - p.e * inv;
-    return {(q.e * p.e - qp) * inv, p.x + q.x * c, p.y + q.y * c, p.z + q.z * c};
-}
-
-// t range of a 2->2 block (Eq. t_invariant_theta): t = A + B cos(theta); the root of larger
-// magnitude directly, the other from t+ t- =
-//   (m1^2 - mA^2)(m2^2 - mB^2) + (m1^2 mB^2 - m2^2 mA^2)(m1^2 - m2^2 - mA^2 + mB^2)/s.
-__device__ __forceinline__ void t_range(double s, double mA2, double mB2, double m1, double m2,
-                                        double& tabs_min, double& tabs_max, double& B) {
-    double m12 = m1 * m1, m22 = m2 * m2;
-    double inv2s = 0.5 / s;
-    double A = mA2 + m12 - (s + mA2 - mB2) * (s + m12 - m22) * inv2s;
-    B = sqrt(kallen(s, mA2, mB2) * kallen_m(s, m1, m2)) * inv2s;
-    double prod = (m12 - mA2) * (m22 - mB2) + (m12 * mB2 - m22 * mA2) * (m12 - m22 - mA2 + mB2) / s;
-    const bool a_nonpos = nonpos_bits(A);       // A <= 0, on the bits
-    double big = a_nonpos ? A - B : A + B;      // root without cancellation
-    double small = !is_zero(big) ? prod / big : 0.0;
-    double tplus = a_nonpos ? small : big;      // closest to zero
-    double tminus = a_nonpos ? big : small;
-    tabs_min = -tplus;
-    tabs_max = -tminus;
-}
 // Sums and products with a term that may be the constant zero of a compiled channel (massless legs):
 // x + 0 and x * 0 do not fold under IEEE rules, a select on the bits of a constant does.
 __device__ __forceinline__ double add_z(double a, double b) { return is_zero(b) ? a : (is_zero(a) ? b : __dadd_rn(a, b)); }
 __device__ __forceinline__ double sub_z(double a, double b) { return is_zero(b) ? a : (is_zero(a) ? -b : __dadd_rn(a, -b)); }
 __device__ __forceinline__ double mul_z(double a, double b) { return is_zero(a) || is_zero(b) ? 0.0 : __dmul_rn(a, b); }
 
-// kallen(x, y, z) of the incoming legs of a 2->2 block with every rounding spelled out
+// Kallen lambda(x, y, z) = (x - y - z)^2 - 4 y z (x >= 0) of the incoming legs of a 2->2 block, without cancellation
+// and with every rounding spelled out:
+//   y, z >= 0: (x - (sqrt y + sqrt z)^2)(x - (sqrt y - sqrt z)^2)
+//   y, z <= 0: x^2 + 2x(|y| + |z|) + (|y| - |z|)^2  (space-like legs of a t-chain)
+//   mixed:     (x - y - z)^2 - 4 y z                (-4yz >= 0)
+// clamped at zero.  The branches are taken on the bit patterns (integer ALU); y = z = 0 (two massless legs)
+// is x^2.
 __device__ __forceinline__ double kallen_in(double x, double y, double z) {
     double l;
     if (is_zero(y) && is_zero(z)) {
@@ -253,7 +184,10 @@ __device__ __forceinline__ double kallen_in(double x, double y, double z) {
     return pos_bits(l) ? l : 0.0;
 }
 
-// The t range for the forward kernels, with what the block itself needs of it: the Kallen functions of
+// t range of a 2->2 block (Eq. t_invariant_theta): t = A + B cos(theta); the root of larger
+// magnitude directly, the other from t+ t- =
+//   (m1^2 - mA^2)(m2^2 - mB^2) + (m1^2 mB^2 - m2^2 mA^2)(m1^2 - m2^2 - mA^2 + mB^2)/s.
+// With it goes what the block itself needs: the Kallen functions of
 // the incoming and outgoing legs and B.  Every rounding is spelled out (no contraction is left to the
 // compiler): the |t| map and the block evaluate it separately, and the distance |t| - |t|_min must be
 // taken from the very bound that |t| was built on.
