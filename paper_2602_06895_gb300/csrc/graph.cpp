@@ -1141,6 +1141,7 @@ struct ps_program_s {
     void* jit_fn = nullptr;  // the compiled kernel (PS_PROGRAM_JIT), else the interpreter runs
     size_t jit_smem = 0;
     int jit_grid = 0;
+    int jit_tiles = 1;       // tiles a CTA of the compiled kernel runs side by side
 };
 
 namespace {
@@ -1175,13 +1176,16 @@ void free_device(ps_program p) {
 
 int64_t tiles_of(int64_t n, int block) { return (n + block - 1) / block; }
 
+// CTAs of a map launch
+int map_grid(ps_program p, int64_t n_tiles) {
+    const int64_t ctas = p->jit_fn ? tiles_of(n_tiles, p->jit_tiles) : n_tiles;
+    return static_cast<int>(std::min<int64_t>(std::max<int64_t>(ctas, 1), p->jit_fn ? p->jit_grid : p->grid_ctas));
+}
+
 // The map launch of a program: its compiled kernel, else the interpreter.
 int launch_program_map(ps_program p, const ps::LaunchParams& lp, void* stream, std::string* err) {
-    if (p->jit_fn) {
-        const int grid = static_cast<int>(std::min<int64_t>(std::max<int64_t>(lp.n_tiles, 1), p->jit_grid));
-        return ps::jit_launch(p->jit_fn, lp, grid, p->jit_smem, stream, err);
-    }
-    const int grid = static_cast<int>(std::min<int64_t>(std::max<int64_t>(lp.n_tiles, 1), p->grid_ctas));
+    const int grid = map_grid(p, lp.n_tiles);
+    if (p->jit_fn) return ps::jit_launch(p->jit_fn, lp, grid, p->jit_smem, stream, err);
     return ps::launch_map(lp, grid, p->smem, stream, err);
 }
 
@@ -1195,6 +1199,7 @@ int fill_launch(ps_program p, const int* chans, const int64_t* counts, int n, co
     lp->smem_imm = p->max_imm;
     lp->smem_grid = p->max_grid;
     lp->smem_slots = p->max_slots;
+    lp->cta_tiles = p->jit_tiles;
     lp->code = p->d_code;
     lp->imm = p->d_imm;
     lp->grid = p->d_grid;
@@ -1386,18 +1391,20 @@ int ps_program_create(const ps_graph* graphs, int n_ch, const ps_options* opt, i
     }
     if (p->opt.flags & PS_PROGRAM_JIT) {  // the compiled kernel: VEGAS grid and reduction scratch in shared memory
         // a requested CTA count also caps the compiled kernel's registers so that many CTAs fit
-        const int min_blocks = std::min(p->opt.ctas_per_sm, 2048 / p->block);
-        st = ps::jit_prepare(p->ch, p->block, min_blocks, p->opt.precision == PS_PRECISION_MIXED, device, &p->jit_fn,
-                             &err);
+        const bool mixed = p->opt.precision == PS_PRECISION_MIXED;
+        const int min_blocks = ps::jit_min_blocks(p->ch.size(), mixed, p->block, p->opt.ctas_per_sm);
+        p->jit_tiles = ps::jit_cta_tiles(p->ch.size(), mixed, p->block, min_blocks, p->max_grid);
+        st = ps::jit_prepare(p->ch, p->block, min_blocks, mixed, p->jit_tiles, device, &p->jit_fn, &err);
         int jit_per_sm = 0;
-        p->jit_smem = (static_cast<size_t>(p->max_grid) + 4 * (p->block / 32)) * sizeof(double);
-        if (st == PS_OK) st = ps::jit_occupancy(p->jit_fn, p->block, p->jit_smem, &jit_per_sm);
+        p->jit_smem = (p->jit_tiles > 1 ? static_cast<size_t>(p->jit_tiles) * ps::jit_group_doubles(p->max_grid, p->block)
+                                        : static_cast<size_t>(p->max_grid) + 4 * (p->block / 32)) * sizeof(double);
+        if (st == PS_OK) st = ps::jit_occupancy(p->jit_fn, p->block * p->jit_tiles, p->jit_smem, &jit_per_sm);
         if (st != PS_OK || jit_per_sm < 1) {
             free_device(p);
             delete p;
             return fail(st != PS_OK ? st : PS_ERR_CAPACITY, st != PS_OK ? err : "compiled kernel does not fit on an SM");
         }
-        const int jit_want = p->opt.ctas_per_sm > 0 ? p->opt.ctas_per_sm : 16;
+        const int jit_want = p->opt.ctas_per_sm > 0 ? std::max(1, p->opt.ctas_per_sm / p->jit_tiles) : 16;
         p->jit_grid = p->sm_count * std::min(jit_per_sm, jit_want);
     }
     *out = p;
@@ -1492,8 +1499,7 @@ int ps_exec_create(ps_program p, const int64_t* events, const ps_out_buffers* ou
     if (st != PS_OK) { delete e; return st; }
     e->lp.r = nullptr;
     e->stats = p->d_stats;
-    e->grid = static_cast<int>(
-        std::min<int64_t>(std::max<int64_t>(e->lp.n_tiles, 1), p->jit_fn ? p->jit_grid : p->grid_ctas));
+    e->grid = map_grid(p, e->lp.n_tiles);
     DeviceGuard dg(p->device);
     cudaStream_t cs;
     st = cuda_check(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking), "cudaStreamCreate");
@@ -1703,8 +1709,9 @@ int ps_jit_check(const ps_graph* graphs, int n_ch, const ps_options* opt, char* 
     }
     std::vector<char> cubin;
     std::string lg;
-    const int min_blocks = opt ? std::min(opt->ctas_per_sm, 2048 / block) : 0;
-    int st = ps::jit_build(ch, block, min_blocks, mixed, &cubin, &lg);
+    const int min_blocks = ps::jit_min_blocks(ch.size(), mixed, block, opt ? opt->ctas_per_sm : 0);
+    const int tiles = ps::jit_cta_tiles(ch.size(), mixed, block, min_blocks, ps::kTrigDoubles);
+    int st = ps::jit_build(ch, block, min_blocks, mixed, tiles, &cubin, &lg);
     if (log_bytes > 0) {
         std::snprintf(log, log_bytes, "%s", lg.c_str());
     }

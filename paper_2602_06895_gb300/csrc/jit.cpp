@@ -283,9 +283,18 @@ const char* kChanParams =
     "(const ps::LaunchParams& lp, const ps::ChannelLaunch& C, int64_t ev, int64_t local, bool active, "
     "double* s_grid, unsigned long long* cut)";
 
-std::string kernel_source(int block, int min_blocks) {
-    const std::string bounds =
-        std::to_string(block) + (min_blocks > 0 ? ", " + std::to_string(min_blocks) : std::string());
+std::string kernel_source(int block, int min_blocks, int tiles) {
+    const std::string bounds = std::to_string(block * tiles) +
+                               (min_blocks > 0 ? ", " + std::to_string(min_blocks / tiles) : std::string());
+    const std::string t = std::to_string(tiles);
+    if (tiles > 1)
+        return "extern \"C\" __global__ void __launch_bounds__(" + bounds +
+               ") ps_jit_map(const __grid_constant__ ps::LaunchParams lp) {\n"
+               "    extern __shared__ __align__(16) double smem[];\n"
+               "    double* part = smem + threadIdx.x / lp.block * ps::jit_group_doubles(lp.smem_grid, lp.block);\n"
+               "    ps::dev::CompiledPolicy<psjit::kMix, psjit::Events, " + t + "> pol{lp, part};\n"
+               "    ps::dev::map_tiles<" + t + ">(lp, pol, part + (lp.smem_grid - ps::kTrigDoubles + 1) / 2);\n"
+               "}\n";
     return "extern \"C\" __global__ void __launch_bounds__(" + bounds +
            ") ps_jit_map(const __grid_constant__ ps::LaunchParams lp) {\n"
            "    extern __shared__ __align__(16) double smem[];\n"
@@ -301,7 +310,7 @@ std::string prologue(bool mixed) {
 }  // namespace
 
 // The CUDA source of a compiled program (all channels, one precision, one block size).
-std::string jit_source(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed) {
+std::string jit_source(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, int tiles) {
     std::string s = prologue(mixed);
     for (size_t c = 0; c < ch.size(); ++c) s += imm_source(ch[c], c);
     s += "struct Events {\n"
@@ -313,13 +322,14 @@ std::string jit_source(const std::vector<Compiled>& ch, int block, int min_block
         s += "            case " + std::to_string(c) + ": {\n" + channel_body(ch[c], c, mixed) + "            }\n";
     }
     s += "        }\n        return 0.0;\n    }\n};\n}  // namespace psjit\n\n";
-    return s + kernel_source(block, min_blocks);
+    return s + kernel_source(block, min_blocks, tiles);
 }
 
 // The split form of a large program: one unit per channel, each defining the channel's event as
 // an external device function, and a kernel unit that dispatches on the channel. The units are
 // compiled separately (in parallel) as relocatable code and linked into one kernel.
-std::vector<std::string> jit_sources_split(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed) {
+std::vector<std::string> jit_sources_split(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed,
+                                           int tiles) {
     std::vector<std::string> units;
     std::string k = prologue(mixed) + "}  // namespace psjit\n";
     for (size_t c = 0; c < ch.size(); ++c)
@@ -332,7 +342,8 @@ std::vector<std::string> jit_sources_split(const std::vector<Compiled>& ch, int 
     for (size_t c = 0; c < ch.size(); ++c)
         k += "            case " + std::to_string(c) + ": return psjit_channel_" + std::to_string(c) +
              "(lp, C, ev, local, active, s_grid, cut);\n";
-    k += "        }\n        return 0.0;\n    }\n};\n}  // namespace psjit\n\n" + kernel_source(block, min_blocks);
+    k += "        }\n        return 0.0;\n    }\n};\n}  // namespace psjit\n\n" +
+         kernel_source(block, min_blocks, tiles);
     units.push_back(k);
     for (size_t c = 0; c < ch.size(); ++c) {
         std::string u = prologue(mixed) + imm_source(ch[c], c) + "}  // namespace psjit\n\n";
@@ -404,6 +415,23 @@ bool split_program(size_t n_ch, bool mixed) {
     return n_ch > static_cast<size_t>(mixed ? kJitInlineMixed : kJitInlineChannels);
 }
 
+}  // namespace
+
+int jit_min_blocks(size_t n_ch, bool mixed, int block, int ctas_per_sm) {
+    if (ctas_per_sm <= 0 && mixed && split_program(n_ch, mixed)) return std::max(1, 512 / block);
+    return std::min(ctas_per_sm, 2048 / block);
+}
+
+int jit_cta_tiles(size_t n_ch, bool mixed, int block, int min_blocks, int smem_grid) {
+    if (!mixed || n_ch < static_cast<size_t>(kJitTilesFrom) || block >= 256 || 256 % block != 0) return 1;
+    const int tiles = 256 / block;
+    if (min_blocks % tiles != 0 || min_blocks / tiles < 2 || min_blocks < 4) return 1;
+    // every group keeps its own grid; the launch does not ask for more than the default 48 KiB
+    if (tiles * jit_group_doubles(smem_grid, block) * sizeof(double) > 48 * 1024) return 1;
+    return tiles;
+}
+
+namespace {
 // nvJitLink: relocatable cubins -> one executable cubin for sm_103a (host only).
 int link_cubins(const std::vector<std::vector<char>>& bins, std::vector<char>* cubin, std::string* log) {
     nvJitLinkHandle h;
@@ -457,7 +485,7 @@ int register_cap(int block, int min_blocks) {
     return std::max(32, std::min(255, regs));
 }
 
-Plan make_plan(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed) {
+Plan make_plan(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, int tiles) {
     Plan p;
     p.split = split_program(ch.size(), mixed);
     if (p.split) {
@@ -469,11 +497,11 @@ Plan make_plan(const std::vector<Compiled>& ch, int block, int min_blocks, bool 
         int slots = 0;
         for (const Compiled& c : ch) slots = std::max(slots, c.n_slots);
         if (!mixed && min_blocks <= 0 && slots <= 64) p.max_regs = register_cap(128, 3);
-        p.units = jit_sources_split(ch, block, min_blocks, mixed);
+        p.units = jit_sources_split(ch, block, min_blocks, mixed, tiles);
         for (const std::string& u : p.units) p.key += u + "\n// ---- unit\n";
         p.key += "// maxrregcount " + std::to_string(p.max_regs) + "\n";
     } else {
-        p.units = {jit_source(ch, block, min_blocks, mixed)};
+        p.units = {jit_source(ch, block, min_blocks, mixed, tiles)};
         p.key = p.units[0];
     }
     return p;
@@ -532,9 +560,9 @@ int build_plan(const Plan& p, std::vector<char>* cubin, std::string* log) {
 }
 }  // namespace
 
-int jit_build(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, std::vector<char>* cubin,
+int jit_build(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, int tiles, std::vector<char>* cubin,
               std::string* log) {
-    return build_plan(make_plan(ch, block, min_blocks, mixed), cubin, log);
+    return build_plan(make_plan(ch, block, min_blocks, mixed, tiles), cubin, log);
 }
 
 namespace {
@@ -585,7 +613,7 @@ std::map<std::pair<int, std::string>, CUfunction_t> g_cache;  // (device, source
 }  // namespace
 
 // Compile (or find in the cache) the program's kernel on the current device.
-int jit_prepare(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, int device, void** fn,
+int jit_prepare(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, int tiles, int device, void** fn,
                 std::string* err) {
     for (const Compiled& C : ch)
         if (!all_finite(C.imm)) {
@@ -597,7 +625,7 @@ int jit_prepare(const std::vector<Compiled>& ch, int block, int min_blocks, bool
         *err = d.why;
         return PS_ERR_CUDA;
     }
-    const Plan plan = make_plan(ch, block, min_blocks, mixed);
+    const Plan plan = make_plan(ch, block, min_blocks, mixed, tiles);
     std::lock_guard<std::mutex> lock(g_cache_mu);
     auto key = std::make_pair(device, plan.key);
     auto it = g_cache.find(key);
@@ -629,11 +657,15 @@ int jit_occupancy(void* fn, int block, size_t smem, int* per_sm) {
     return PS_OK;
 }
 
+namespace {
+unsigned cta_threads(const LaunchParams& lp) { return static_cast<unsigned>(lp.block * std::max(1, lp.cta_tiles)); }
+}  // namespace
+
 int jit_launch(void* fn, const LaunchParams& lp, int grid, size_t smem, void* stream, std::string* err) {
     if (lp.n_tiles == 0) return PS_OK;
     Driver& d = driver();
     void* args[] = {const_cast<LaunchParams*>(&lp)};
-    const int r = d.launchKernel(fn, static_cast<unsigned>(grid), 1, 1, static_cast<unsigned>(lp.block), 1, 1,
+    const int r = d.launchKernel(fn, static_cast<unsigned>(grid), 1, 1, cta_threads(lp), 1, 1,
                                  static_cast<unsigned>(smem), stream, args, nullptr);
     if (r != 0) {
         *err = "compiled kernel launch failed (driver error " + std::to_string(r) + ")";
@@ -663,7 +695,7 @@ int jit_node_set(void* exec, void* node, void* fn, const LaunchParams& lp, int g
     kp.func = static_cast<CUfunction>(fn);
     kp.gridDimX = static_cast<unsigned>(grid);
     kp.gridDimY = kp.gridDimZ = 1;
-    kp.blockDimX = static_cast<unsigned>(lp.block);
+    kp.blockDimX = cta_threads(lp);
     kp.blockDimY = kp.blockDimZ = 1;
     kp.sharedMemBytes = static_cast<unsigned>(smem);
     kp.kernelParams = args;  // copied by the call

@@ -15,6 +15,15 @@ constexpr int kOpOutput = 1000;  // pseudo-op closing each channel's byte-code
 constexpr int kTrigN = 256;
 constexpr int kTrigDoubles = 2 * kTrigN;
 
+// Shared-memory doubles of one group of a compiled mixed kernel that runs several tiles a CTA: the VEGAS grid in
+// floats (no azimuth table) and the records of the tile's statistics, in whole 16 bytes.
+#if defined(__CUDACC__) || defined(__CUDACC_RTC__)
+__host__ __device__
+#endif
+constexpr int jit_group_doubles(int smem_grid, int block) {
+    return ((smem_grid - kTrigDoubles + 1) / 2 + 4 * (block / 32) + 1) & ~1;
+}
+
 // ---------------------------------------------------------------- launch description
 struct ChannelLaunch {
     int32_t code_off, code_len;    // ints in the code buffer
@@ -33,7 +42,7 @@ struct ChannelLaunch {
 
 struct LaunchParams {
     int32_t n_ch;
-    int32_t block;                 // threads per CTA = events per tile
+    int32_t block;                 // events per tile = threads per CTA (of a compiled kernel: per group)
     int32_t smem_code_ints, smem_imm, smem_grid, smem_slots;  // per-CTA staging sizes
     int64_t n_tiles;
     const int32_t* code;
@@ -51,6 +60,7 @@ struct LaunchParams {
     void* alpha;
     int64_t ld;
     int32_t mixed;
+    int32_t cta_tiles;             // a compiled kernel's groups per CTA, one tile each (0 counts as 1)
     // scratch and program state
     double* tile_partials;         // [n_tiles][4]
     double* hist;                  // VEGAS histograms (program-owned), or nullptr

@@ -1326,24 +1326,32 @@ __device__ __forceinline__ double store_outputs(const Fr& f, const int32_t* od, 
 // `block` events over all channels (tile -> channel by the prefix sums in the parameters), a
 // channel change stages the channel's shared data (pol.stage), every thread evaluates one event
 // (pol.event -> weight), then the tile's partial sums.  (The VEGAS training histogram is a separate
-// pass over the stored weights, in a fixed order.)
-template <class Policy>
+// pass over the stored weights, in a fixed order.)  With kTiles > 1 a CTA is kTiles groups of `block` threads with a
+// tile and shared memory each, which meet at the tile's barriers.
+template <int kTiles = 1, class Policy>
 __device__ __forceinline__ void map_tiles(const LaunchParams& lp, Policy& pol, double* s_red) {
     const int B = lp.block;
-    const int tid = threadIdx.x;
+    const int group = kTiles > 1 ? threadIdx.x / B : 0;
+    const int tid = threadIdx.x - group * B;
     int cur = -1;
-    for (int64_t tile = blockIdx.x; tile < lp.n_tiles; tile += gridDim.x) {
+    for (int64_t first = kTiles * static_cast<int64_t>(blockIdx.x); first < lp.n_tiles;
+         first += kTiles * static_cast<int64_t>(gridDim.x)) {
+        // a group past the last tile goes through that tile's motions, with no event active
+        const bool has = kTiles == 1 || first + group < lp.n_tiles;
+        const int64_t tile = has ? first + group : lp.n_tiles - 1;
         int c = 0;
         while (c + 1 < lp.n_ch && tile >= lp.ch[c + 1].tile_begin) ++c;
         const ChannelLaunch& C = lp.ch[c];
-        if (c != cur) {
+        bool change = c != cur;
+        if constexpr (kTiles > 1) change = __syncthreads_or(change) != 0;  // every group takes part in the barriers
+        if (change) {
             __syncthreads();
             pol.stage(c, C);
             __syncthreads();
             cur = c;
         }
         const int64_t local = (tile - C.tile_begin) * B + tid;
-        const bool active = local < C.n_events;
+        const bool active = has && local < C.n_events;
         const int64_t ev = C.ev_offset + local;
         double w = pol.event(c, C, ev, local, active);
         if (!active) w = 0.0;
@@ -1378,7 +1386,7 @@ __device__ __forceinline__ void map_tiles(const LaunchParams& lp, Policy& pol, d
             s_red[4 * warp + 2] = sum;
         }
         __syncthreads();
-        if (tid == 0) {
+        if (tid == 0 && has) {
             double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
             for (int k = 0; k < B / 32; ++k) {
                 a0 += s_red[4 * k];
@@ -1397,21 +1405,24 @@ __device__ __forceinline__ void map_tiles(const LaunchParams& lp, Policy& pol, d
 
 // A compiled program's policy: the VEGAS grid is the only shared data; the generated `Events`
 // evaluates channel c's instruction list on a register frame.
-template <bool kMix, class Events>
+template <bool kMix, class Events, int kTiles = 1>
 struct CompiledPolicy {
+    static constexpr int kGridAt = kTiles > 1 ? 0 : kTrigDoubles;  // after the azimuth table, where there is one
+    static_assert(kMix || kTiles == 1, "the FP64 form keeps its azimuth table, one tile a CTA");
     const LaunchParams& lp;
     double* s_grid;
     __device__ __forceinline__ void stage(int c, const ChannelLaunch& C) {
-        double* g = s_grid + kTrigDoubles;  // after the azimuth table
+        double* g = s_grid + kGridAt;
         if constexpr (kMix) {
-            stage_grid(reinterpret_cast<float*>(g), lp.grid + C.grid_off, C.vdims, C.vbins, threadIdx.x, lp.block);
+            const int tid = kTiles > 1 ? threadIdx.x % lp.block : threadIdx.x;
+            stage_grid(reinterpret_cast<float*>(g), lp.grid + C.grid_off, C.vdims, C.vbins, tid, lp.block);
         } else {
             stage_trig(s_grid, threadIdx.x, lp.block);
             stage_grid(g, lp.grid + C.grid_off, C.vdims, C.vbins, threadIdx.x, lp.block);
         }
     }
     __device__ __forceinline__ double event(int c, const ChannelLaunch& C, int64_t ev, int64_t local, bool active) {
-        return Events::run(c, lp, C, ev, local, active, s_grid + kTrigDoubles, lp.status + 1);
+        return Events::run(c, lp, C, ev, local, active, s_grid + kGridAt, lp.status + 1);
     }
 };
 

@@ -103,17 +103,31 @@ void count_launches(int n);
 // cached kernel on the current device, its occupancy and its launch.
 // min_blocks > 0: the kernel is compiled so that that many CTAs of `block` threads fit on an SM
 // (launch bounds; the split form's channel units get the matching register cap).
-std::string jit_source(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed);
+std::string jit_source(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, int tiles);
+// Tiles a CTA of a compiled program runs side by side: several for a mixed program of several channels that is asked
+// to fit four CTAs or more on an SM, as long as two CTAs and 256 threads remain.  Such a program's code is
+// straight-line and long (2->8: ~10^4 instructions an event), instruction fetch bounds it, and warps that leave a
+// barrier together share what they fetch: 128 threads x 4 CTAs took 4.95 ms per 2^22 2->8 events, 2 x 128 threads x
+// 2 CTAs, with the same registers and warps, 4.28 ms (64 x 8: 7.53 and 4.26 ms; 2->5, 6e6 events, 128 x 4: 4.53 and
+// 4.32 ms).  Two CTAs of 128 threads, 8 warps an SM, gain nothing (2->8: 6.12 and 6.20 ms).
+constexpr int kJitTilesFrom = 3;  // channels
+// The CTAs an SM is to hold: those requested; when none are, for a split mixed program, as many as hold 512 threads
+// at 128 registers (2->8 at 128 threads: 6.25 ms with the registers the compiler takes, 4.29 ms with 128).  A
+// program in one unit does better with the compiler's own choice (2->5: 4.09 ms against 4.32 ms capped; three 2->8
+// channels, 2^21 events: 2.12 against 2.29 ms).
+int jit_min_blocks(size_t n_ch, bool mixed, int block, int ctas_per_sm);
+int jit_cta_tiles(size_t n_ch, bool mixed, int block, int min_blocks, int smem_grid);
 int jit_compile(const std::string& src, std::vector<char>* cubin, std::string* log, bool relocatable, int max_regs);
 // Programs of more channels than these are compiled one unit per channel, in parallel, and linked: one
 // unit of all channels compiles in time that grows faster than the channel count.  FP64 units are
 // longer (six 2->5 channels: 14.5 s as one unit, 2.3 s as six, the kernel 5% slower), mixed ones shorter.
 constexpr int kJitInlineChannels = 2, kJitInlineMixed = 6;
-std::vector<std::string> jit_sources_split(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed);
+std::vector<std::string> jit_sources_split(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed,
+                                           int tiles);
 // The program's kernel as one executable cubin: a single unit, or the split units linked.
-int jit_build(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, std::vector<char>* cubin,
-              std::string* log);
-int jit_prepare(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, int device, void** fn,
+int jit_build(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, int tiles,
+              std::vector<char>* cubin, std::string* log);
+int jit_prepare(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, int tiles, int device, void** fn,
                 std::string* err);
 int jit_occupancy(void* fn, int block, size_t smem, int* per_sm);
 int jit_launch(void* fn, const LaunchParams& lp, int grid, size_t smem, void* stream, std::string* err);
