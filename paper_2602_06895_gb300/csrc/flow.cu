@@ -1455,8 +1455,8 @@ __device__ __forceinline__ void hidden_columns(const uint32_t (&v)[32], const fl
 }
 // The warpgroup's 64 hidden columns: the second half's accumulators are on their way from TMEM while the first
 // half's SiLUs run (1708 -> 1687 us for 2^20 events through six layers; loading each half and waiting for it before its
-// own SiLUs exposed the load twice a layer).  The TMEM loads are warp-collective (.sync.aligned): every lane of the warp executes them,
-// whatever `store` is.
+// own SiLUs exposed the load twice a layer).  The TMEM loads are warp-collective (.sync.aligned): every lane of the
+// warp executes them, whatever `store` is.
 template <bool kStore>
 __device__ __forceinline__ void hidden_epilogue(uint32_t taddr, const float* bias, bf16* act, int row, int c0,
                                                 bool store = false, float* zg = nullptr, bf16* ag = nullptr) {
@@ -1974,7 +1974,8 @@ void free_flow(ps_flow f) {
                     static_cast<void*>(f->logdet), static_cast<void*>(f->G), static_cast<void*>(f->Gb),
                     static_cast<void*>(f->dA), static_cast<void*>(f->dZ), static_cast<void*>(f->dZb), static_cast<void*>(f->dAb),
                     static_cast<void*>(f->dIn), static_cast<void*>(f->gX), static_cast<void*>(f->gXn),
-                    static_cast<void*>(f->wtot), static_cast<void*>(f->cw), static_cast<void*>(f->lterm), static_cast<void*>(f->colpart), static_cast<void*>(f->scal),
+                    static_cast<void*>(f->wtot), static_cast<void*>(f->cw), static_cast<void*>(f->lterm),
+                    static_cast<void*>(f->colpart), static_cast<void*>(f->scal),
                     static_cast<void*>(f->gen_X), static_cast<void*>(f->gen_ld),
                     static_cast<void*>(f->gen_status)})
         cudaFree(q);

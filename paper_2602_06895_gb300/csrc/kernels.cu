@@ -34,6 +34,7 @@ static unsigned long long g_launches = 0;
 // shared memory; an event runs the byte-code on the thread's column of the slot file.
 template <bool kMix>
 struct InterpPolicy {
+    static constexpr bool kTwoJoins = false;  // map_tiles
     const LaunchParams& lp;
     dev::Frame f;
     int32_t* s_code;
