@@ -15,7 +15,8 @@ reaches the Grace memory over NVLink-C2C), timed on the host clock with the per-
 channel sums; the copy-engine form (HBM, then a copy on a second stream) is reported beside it.
 
 Every timed map runs the program compiled at creation (NVRTC, the slot file in registers;
-programs of more than six channels compiled one unit per channel and linked); `--no-jit` runs
+FP64 programs of more than two channels, mixed ones of more than six, compiled one unit per
+channel and linked); `--no-jit` runs
 the interpreter kernel instead, and the main leg reports the interpreter's time beside it.
 Compile times fall outside the timed regions.
 
@@ -44,52 +45,44 @@ WORKLOAD = ("hadronic 2->4 W W at sqrt(S)=13 TeV: 1/tau shat map, r_to_x1x2, 2 B
             "massless, f(x)=x^-1.1(1-x)^3, 8-dim VEGAS x 64 bins adapted 10x1e6 then frozen, 1e7 events/step, FP64")
 # Algorithmic output bytes of one event: 6 momenta x 4 x 8 + x1 + x2 + w.
 BYTES_PER_EVENT = 6 * 4 * 8 + 8 + 8 + 8
-# FP64 floating-point operations executed per event by the map kernel (DFMA = 2, DADD/DMUL = 1):
-# 2 x 438.2 + 140.6 + 233.7 from the ncu instruction counters of this kernel on this workload
-# (profiles/ps_map_kernel_ww_2to4.md).
-FP64_FLOP_PER_EVENT = 1250.7
+# FP64 floating-point operations executed per event by the interpreter's map kernel (DFMA = 2, DADD/DMUL = 1):
+# 2 x 188.8 + 77.5 + 153.5 from the ncu instruction counters of this kernel on this workload
+# (profiles/fp64_pipe_probes.md).
+FP64_FLOP_PER_EVENT = 608.4
 # DRAM traffic per event from the same capture (read + write, 2e6-event launch), scaled to a launch.
-DRAM_BYTES_PER_EVENT = 186.0
+DRAM_BYTES_PER_EVENT = 185.5
 # FP64 peak of a GB300: 1.25 TFLOP/s nominal (152 SMs x 2 DFMA/clk x ~2.07 GHz) -- the ALU peak
 # derived from the unit counts and clocks; no measured FP64 peak is provided.
 FP64_PEAK_GFLOPS = 1250.0
 # The binding resource is the FP64 pipe: 2 FP64 instructions per clock per SM, whether DFMA, DADD
 # or DMUL, i.e. 152 x 2 x 2.07 GHz = 629.3 G instructions/s.  FP64 arithmetic instructions per
-# event of the map kernel from the same ncu capture: DFMA + DADD + DMUL = 438.2 + 140.6 + 233.7.
-FP64_INSTR_PER_EVENT = 812.5
+# event of the interpreter's kernel from the same ncu capture: DFMA + DADD + DMUL = 188.8 + 77.5 + 153.5.
+FP64_INSTR_PER_EVENT = 419.7
 FP64_PEAK_GINSTR = 152 * 2 * 2.07
 # The same counters for the compiled program's kernel (ps_jit_map) on this workload, from its own
-# ncu capture (profiles/ps_jit_map_ww_2to4.md): DFMA 405.6 + DADD 113.6 + DMUL 197.6 = 716.8 FP64
-# arithmetic instructions (1122.4 flops) and 185.9 DRAM bytes per event; FP64 pipe 85.4 % active.
-# Re-captured on the current build (the Kallen function of decays and 2->2 blocks taken from the
-# masses, the per-tile statistics with six FP64 instructions per event, bins, maxima and sign
-# tests on the integer ALU, one exponential for both parton densities, x2 = tau / x1, the decay
-# daughters boosted with one dot product, the VEGAS bin widths staged with the grid, the
-# collider's 1/S folded, the azimuths from a 256-point table and short Taylor series, the
-# Breit-Wigner map's tangent from a double-double table and its regions without branches;
-# profiles/fp64_pipe_probes.md): DFMA 331.9 + DADD 101.6 + DMUL 209.6 = 643.0 (974.9 flops),
-# 676.7 FP64-pipe instructions in all (688.5 in warp-issue slots x 32: lanes 0.983 busy),
-# 185.3 DRAM bytes per event, pipe active 0.845 of the elapsed cycles -- the FP64 issue probe's
-# saturating loop reaches 0.84.
-COMPILED_COUNTERS = {"instr": 643.0, "flops": 974.9, "dram": 185.3, "pipe": 0.845, "pipe_instr": 676.7}
+# ncu capture (profiles/fp64_pipe_probes.md): DFMA 178.3 + DADD 63.7 + DMUL 136.7 = 378.7 FP64
+# arithmetic instructions (557.0 flops), 380.8 FP64-pipe instructions in all (393.0 in warp-issue slots
+# x 32: lanes 0.97 busy), 185.3 DRAM bytes per event, pipe active 0.853 of the elapsed cycles -- the
+# FP64 issue probe's saturating loop reaches 0.84.  (643.0, 676.7 and 688.5 while divisions, roots and the
+# maps' functions were CUDA's own: they start from FP32 seeds and tables now.)
+COMPILED_COUNTERS = {"instr": 378.7, "flops": 557.0, "dram": 185.3, "pipe": 0.853, "pipe_instr": 380.8}
 INTERPRETER_COUNTERS = {"instr": FP64_INSTR_PER_EVENT, "flops": FP64_FLOP_PER_EVENT, "dram": DRAM_BYTES_PER_EVENT,
-                        "pipe": 0.854}
+                        "pipe": 0.765, "pipe_instr": 423.7}
 # FP64 arithmetic instructions (DFMA + DADD + DMUL) per event of the 24-channel 2->8 workload, from
-# the ncu captures of one 2^20-event launch: the compiled program on the current build
-# (profiles/fp64_pipe_probes.md: 2451.3 + 1058.3 + 895.5); the interpreter's from an earlier build
-# (profiles/ps_map_kernel_c5_2to8.md, before the mass-based Kallen function; an upper bound).
-C5_FP64_INSTR_PER_EVENT = {"compiled": 4405.0, "interpreter": 6559.0}
+# the ncu captures of one 2^20-event launch (profiles/fp64_pipe_probes.md): the compiled program 864.6 +
+# 937.3 + 585.9, the interpreter 1170.0 + 1918.6 + 996.3.
+C5_FP64_INSTR_PER_EVENT = {"compiled": 2387.8, "interpreter": 4084.8}
 # The same for the compiled six-channel 2->5 program, from one 2e6-event launch in the benchmark's
-# channel proportions (profiles/fp64_pipe_probes.md): DFMA 998.1 + DADD 287.0 + DMUL 409.8.
-C3_FP64_INSTR_PER_EVENT = 1694.9
+# channel proportions (profiles/fp64_pipe_probes.md): DFMA 368.9 + DADD 196.2 + DMUL 258.3.
+C3_FP64_INSTR_PER_EVENT = 823.4
 # FP64-pipe instructions in all (arithmetic and conversions) per event of the compiled mixed-precision
 # programs (profiles/fp64_pipe_probes.md): the FP64 pipe's share of the mixed form (with the
-# conversions on the integer ALU, 0.55-0.75 of its cycles: no longer the only bound).
+# conversions on the integer ALU, 0.54-0.78 of its cycles: not the only bound).
 # Launch shapes (threads per CTA, CTAs per SM) the autotuner tries for compiled programs: the
 # CTA count caps the registers (65536 / (threads x CTAs)); the large CTAs keep more warps on the
 # same stretch of a long straight-line program, which the instruction cache rewards.
 JIT_SHAPES = ((128, 2), (128, 3), (128, 4), (256, 1), (256, 2), (256, 3), (512, 1))
-MIXED_FP64_PIPE_PER_EVENT = {"2to4": 61.0, "2to5": 312.6, "2to8": 434.6}
+MIXED_FP64_PIPE_PER_EVENT = {"2to4": 60.9, "2to5": 288.1, "2to8": 435.1}
 # FP64-pipe instructions per call of CUDA's double functions on the GB300, from the ncu counters of
 # ps_fp64_probe's function loops less the empty loop (profiles/fp64_pipe_probes.md); an add or a
 # multiply is one.  They convert the oracle's operation counts into the pipe's work.
