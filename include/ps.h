@@ -235,7 +235,8 @@ int ps_graph_build_channel(const ps_channel_desc* ch, int n_ch, int which, ps_gr
 typedef struct {
     int32_t block_threads; /* events per tile = threads per CTA (multiple of 32, at most 256, or 512
                             * for a compiled program, PS_PROGRAM_JIT; 0 = default 128)         */
-    int32_t ctas_per_sm;   /* resident CTAs requested per SM (0 = as many as fit, up to 4; a
+    int32_t ctas_per_sm;   /* resident CTAs requested per SM (0 = as many as fit, up to 4, or up to the
+                            * launch's tiles where all of them fit at once; a
                             * compiled program, PS_PROGRAM_JIT, caps its registers so that this
                             * many fit, and takes as many as fit when 0; a mixed one of more than six
                             * channels holds 512 threads an SM when 0, and one of more than two may
