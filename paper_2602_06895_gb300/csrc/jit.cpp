@@ -477,12 +477,13 @@ struct Plan {
     std::string key;
 };
 
-// The register cap under which min_blocks CTAs of `block` threads fit on an SM (65536 registers,
-// allocated in steps of 8 per thread), or 0 for no cap.
+// The register cap under which min_blocks CTAs of `block` threads fit on an SM, or 0 for no cap: an SM's registers are
+// four banks of 16384 that its warps go round, allocated in steps of 8 per thread.  The linker refuses channel units
+// beyond it (65536 / threads gave a few registers too many where the warps are no multiple of four).
 int register_cap(int block, int min_blocks) {
     if (min_blocks <= 0) return 0;
-    const int regs = (65536 / (block * min_blocks)) & ~7;
-    return std::max(32, std::min(255, regs));
+    const int per_bank = (block / 32 * min_blocks + 3) / 4;
+    return std::max(32, std::min(255, (16384 / (32 * per_bank)) & ~7));
 }
 
 Plan make_plan(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, int tiles) {
@@ -497,6 +498,10 @@ Plan make_plan(const std::vector<Compiled>& ch, int block, int min_blocks, bool 
         int slots = 0;
         for (const Compiled& c : ch) slots = std::max(slots, c.n_slots);
         if (!mixed && min_blocks <= 0 && slots <= 64) p.max_regs = register_cap(128, 3);
+        // The launch bounds of the kernel unit do not reach the channel units: without the cap of one CTA the link is
+        // refused above 256 threads.
+        const int one = register_cap(block, 1);
+        p.max_regs = p.max_regs > 0 ? std::min(p.max_regs, one) : one;
         p.units = jit_sources_split(ch, block, min_blocks, mixed, tiles);
         for (const std::string& u : p.units) p.key += u + "\n// ---- unit\n";
         p.key += "// maxrregcount " + std::to_string(p.max_regs) + "\n";
