@@ -76,7 +76,7 @@ struct State {
     unsigned long long invalid;
     double t;                           // the result once done
     int done;
-    unsigned int n_list;                // entries of the list
+    unsigned long long n_list;          // weights for the list (it holds no more than its length of them)
     unsigned int ticket;                // blocks of the running kernel that have finished
 };
 
@@ -281,7 +281,8 @@ __global__ void __launch_bounds__(kThreads) k_partials(const double* w, int64_t 
 __global__ void __launch_bounds__(kThreads) k_gather(const double* w, int64_t n, State* st, unsigned long long* list,
                                                      unsigned int list_max) {
     __shared__ unsigned long long buf[kUnroll * kThreads];
-    __shared__ unsigned int cnt, at;
+    __shared__ unsigned int cnt;
+    __shared__ unsigned long long at;
     if (st->done || !st->compact) return;
     const unsigned long long lo = st->lo;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -306,9 +307,10 @@ __global__ void __launch_bounds__(kThreads) k_gather(const double* w, int64_t n,
             if (in) buf[p] = u[k];
         }
         __syncthreads();
-        if (tid == 0) at = cnt ? atomicAdd(&st->n_list, cnt) : 0;
+        if (tid == 0) at = cnt ? atomicAdd(&st->n_list, static_cast<unsigned long long>(cnt)) : 0;
         __syncthreads();
-        const unsigned m = cnt, a = at;
+        const unsigned m = cnt;
+        const unsigned long long a = at;
         for (unsigned i = tid; i < m; i += kThreads)
             if (a + i < list_max) list[a + i] = buf[i];
         __syncthreads();
@@ -330,7 +332,7 @@ __global__ void __launch_bounds__(kThreads) k_pass(const double* w, int64_t n, c
     const unsigned long long lo = st->lo, hi = st->hi;
     const int shift = st->shift;
     const unsigned long long step = 1ULL << shift;
-    const int64_t total = st->compact ? static_cast<int64_t>(min(st->n_list, list_max)) : n;
+    const int64_t total = st->compact ? static_cast<int64_t>(min(st->n_list, static_cast<unsigned long long>(list_max))) : n;
     const unsigned long long* src = st->compact ? list : reinterpret_cast<const unsigned long long*>(w);
     const int64_t chunk = (total + gridDim.x - 1) / gridDim.x;
     const int64_t b0 = blockIdx.x * chunk, b1 = min(total, b0 + chunk);
@@ -432,10 +434,12 @@ __global__ void __launch_bounds__(kThreads) k_pass(const double* w, int64_t n, c
     if (tid != sel) return;
     x.ticket = 0;
     if (x.guess) {
-        // the guessed edge (its own excess not above the target) or the list (cut short) was wrong: from 0, in all weights
+        // the guessed edge (its own excess not above the target) or the list (cut short, also from 0 on: the sample sees
+        // few weights where it meets invalid ones) was wrong: from 0, in all weights
         x.guess = 0;
         const double T = __longlong_as_double(static_cast<long long>(lo));
-        if (lo > 0 && (!(cs[0] - T * static_cast<double>(cc[0]) > x.target) || (x.compact && x.n_list > list_max))) {
+        const bool cut = x.compact && x.n_list > list_max;
+        if (cut || (lo > 0 && !(cs[0] - T * static_cast<double>(cc[0]) > x.target))) {
             x.compact = 0;
             x.lo = 0;
             x.shift = max(0, 56 - __clzll(static_cast<long long>(x.hi)));
