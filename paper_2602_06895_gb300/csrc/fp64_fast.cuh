@@ -132,11 +132,14 @@ __device__ __forceinline__ double rcp(double x) {
     return r;
 }
 __device__ __forceinline__ double div(double a, double b) {
-    // b and a/b in the middle of the range (or a zero)
+    // b and a/b in the middle of the range (or a zero, whose quotient is its product with the seed: the remainder's
+    // sum would lose the sign of -0)
     const uint32_t ea = (hi32(a) >> 20) & 0x7FFu, eb = (hi32(b) >> 20) & 0x7FFu;
-    const bool ok = eb - 64u < 1920u && ((ea - 64u < 1920u && ea - eb + 900u < 1800u) || (hi32(a) << 1 | lo32(a)) == 0u);
+    const bool zero = (hi32(a) << 1 | lo32(a)) == 0u;
+    const bool ok = eb - 64u < 1920u && ((ea - 64u < 1920u && ea - eb + 900u < 1800u) || zero);
     const double r = rcp_seed(b), q = __dmul_rn(a, r);
     double v = fma(fma(-b, q, a), r, q);
+    if (zero) v = q;
     if (__builtin_expect(!ok, 0)) v = slow_div(a, b);
     return v;
 }
