@@ -33,6 +33,11 @@ static __device__ __noinline__ double slow_sub(double a, double b) { return a - 
 static __device__ __noinline__ double slow_sqrt(double x) { return ::sqrt(x); }
 static __device__ __noinline__ double slow_rsqrt(double x) { return ::rsqrt(x); }
 static __device__ __noinline__ double slow_exp(double x) { return ::exp(x); }
+// exp(v + w) for a correction w of a few ulps of v: e + e w
+static __device__ __noinline__ double slow_exp(double v, double w) {
+    const double e = ::exp(v);
+    return ::isfinite(e) && ::isfinite(w) ? ::fma(e, w, e) : e;
+}
 static __device__ __noinline__ double slow_expm1(double x) { return ::expm1(x); }
 static __device__ __noinline__ double slow_log(double x) { return ::log(x); }
 static __device__ __noinline__ double slow_log1p(double x) { return ::log1p(x); }
@@ -243,7 +248,7 @@ __device__ __forceinline__ double exp(double v, double w) {
     const double r = __dadd_rn(e.r, w);
     const double c = widen(fmaf(e.rf, fmaf(e.rf, 1.0f / 120.0f, 1.0f / 24.0f), 1.0f / 6.0f));
     double x = __dadd_rn(e.t, fma(e.t, fma(__dmul_rn(r, r), fma(r, c, 0.5), r), e.l));
-    if (__builtin_expect(!exp_range(v), 0)) x = slow_exp(v);
+    if (__builtin_expect(!exp_range(v), 0)) x = slow_exp(v, w);
     return x;
 }
 // exp(v) - 1: T - 1 is exact where it cancels (T in [1/2, 2]) and 0 for j = q = 0; the result may be
