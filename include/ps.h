@@ -239,8 +239,8 @@ typedef struct {
                             * launch's tiles where all of them fit at once; a
                             * compiled program, PS_PROGRAM_JIT, caps its registers so that this
                             * many fit, and takes as many as fit when 0; a mixed one of more than six
-                            * channels holds 512 threads an SM when 0, and one of more than two may
-                            * run several of the requested CTAs as one, a tile each)             */
+                            * channels holds 512 threads an SM when 0, and may run several of the
+                            * requested CTAs as one, a tile each)                                */
     int32_t precision;     /* PS_PRECISION_*                                                  */
     int32_t flags;         /* PS_PROGRAM_* bits                                               */
 } ps_options;

@@ -1184,7 +1184,8 @@ int64_t tiles_of(int64_t n, int block) { return (n + block - 1) / block; }
 int map_grid(ps_program p, int64_t n_tiles) {
     if (!p->jit_fn && p->opt.ctas_per_sm <= 0 && n_tiles > p->grid_ctas && n_tiles <= p->grid_fit)
         return static_cast<int>(n_tiles);
-    const int64_t ctas = p->jit_fn ? tiles_of(n_tiles, p->jit_tiles) : n_tiles;
+    // (a compiled kernel of several tiles a CTA spreads a round over the CTAs by halves, map_tiles)
+    const int64_t ctas = tiles_of(n_tiles, p->jit_fn ? std::max(1, p->jit_tiles / 2) : 1);
     return static_cast<int>(std::min<int64_t>(std::max<int64_t>(ctas, 1), p->jit_fn ? p->jit_grid : p->grid_ctas));
 }
 

@@ -423,7 +423,7 @@ int jit_min_blocks(size_t n_ch, bool mixed, int block, int ctas_per_sm) {
 }
 
 int jit_cta_tiles(size_t n_ch, bool mixed, int block, int min_blocks, int smem_grid) {
-    if (!mixed || n_ch < static_cast<size_t>(kJitTilesFrom) || block >= 256 || 256 % block != 0) return 1;
+    if (!mixed || !split_program(n_ch, mixed) || block >= 256 || 256 % block != 0) return 1;
     const int tiles = 256 / block;
     if (min_blocks % tiles != 0 || min_blocks / tiles < 2 || min_blocks < 4) return 1;
     // every group keeps its own grid; the launch does not ask for more than the default 48 KiB

@@ -104,13 +104,13 @@ void count_launches(int n);
 // min_blocks > 0: the kernel is compiled so that that many CTAs of `block` threads fit on an SM
 // (launch bounds; the split form's channel units get the matching register cap).
 std::string jit_source(const std::vector<Compiled>& ch, int block, int min_blocks, bool mixed, int tiles);
-// Tiles a CTA of a compiled program runs side by side: several for a mixed program of several channels that is asked
-// to fit four CTAs or more on an SM, as long as two CTAs and 256 threads remain.  Such a program's code is
-// straight-line and long (2->8: ~10^4 instructions an event), instruction fetch bounds it, and warps that leave a
-// barrier together share what they fetch: 128 threads x 4 CTAs took 4.95 ms per 2^22 2->8 events, 2 x 128 threads x
-// 2 CTAs, with the same registers and warps, 4.28 ms (64 x 8: 7.53 and 4.26 ms; 2->5, 6e6 events, 128 x 4: 4.53 and
-// 4.32 ms).  Two CTAs of 128 threads, 8 warps an SM, gain nothing (2->8: 6.12 and 6.20 ms).
-constexpr int kJitTilesFrom = 3;  // channels
+// Tiles a CTA of a compiled program runs side by side: several for a split mixed program that is asked to fit four CTAs
+// or more on an SM, as long as two CTAs and 256 threads remain.  Such a program's code is straight-line and long (24
+// 2->8 channels: ~10^4 instructions an event each), instruction fetch bounds it, and neighbouring tiles, mostly of one
+// channel, share what they fetch: 128 threads x 4 CTAs took 5.1 ms per 2^22 2->8 events, 2 x 128 threads x 2 CTAs, with
+// the same registers and warps, 4.22 ms (64 x 8: 7.6 and 4.20 ms; 9728 events: 80 and 74 us).  A program in one unit
+// gains nothing (six 2->5 channels, 128 x 4: 6e6 events 4.23 ms with two tiles, 4.19 with one, 38912 events 79 and 65 us).
+// Two CTAs of 128 threads, 8 warps an SM, gain nothing either (2->8: 6.12 and 6.20 ms).
 // The CTAs an SM is to hold: those requested; when none are, for a split mixed program, as many as hold 512 threads
 // at 128 registers (2->8 at 128 threads: 6.25 ms with the registers the compiler takes, 4.29 ms with 128).  A
 // program in one unit does better with the compiler's own choice (2->5: 4.09 ms against 4.32 ms capped; three 2->8
