@@ -20,8 +20,8 @@
 //     once.
 // What bounds it: one read of the weights from HBM and one from L2, and the FP64 pipe in the first (one add per
 // weight, 19 us per 1e7; the maximum and the tests are integer).  1e7 weights, eps = 1e-3: 685 us as eight
-// passes over all weights with per-block histograms combined by one block, 136 us now (eps = 1e-2, where the tail
-// outgrows the list: 771 -> 336 us).
+// passes over all weights with per-block histograms combined by one block, 140 us now; where the tail outgrows the
+// list, eps = 1e-2: 771 -> 216 us, 0.6: 760 -> 532 us (852 with one load in flight a thread and two blocks an SM).
 //
 // The bucket sums are exact integers: a weight m 2^(e-1075) (53-bit significand m, exponent
 // field e) enters its bucket as m 2^(e-E) in units of 2^(E-1075), E the exponent field of the
@@ -59,7 +59,8 @@ constexpr int64_t kSampleFrom = 1 << 20;  // lists from this length on are count
 constexpr int kUnroll = 8;          // loads in flight per thread
 constexpr int kCoarseShift = 50;    // the counting histogram: exponent and two fraction bits
 constexpr int kCoarse = 1 << (63 - kCoarseShift);
-constexpr int kPassGrid = 304;       // two blocks per SM
+constexpr int kPassGrid = 304;       // two blocks per SM, and twice as many from kSampleFrom weights on
+constexpr int kPassUnroll = 4;      // loads in flight per thread of a radix pass
 constexpr int64_t kListMax = 1 << 20;  // weights of the tail list (at most 8 MiB of the workspace)
 constexpr int kSelPerThread = 8;    // events per thread in the select kernels
 constexpr int kSelBlock = kThreads * kSelPerThread;
@@ -129,7 +130,7 @@ __global__ void __launch_bounds__(256) k_zero(State* st, unsigned int* coarse, u
 __global__ void __launch_bounds__(kThreads) k_partials(const double* w, int64_t n, double eps, double* part,
                                                        unsigned int* coarse, unsigned int list_max, State* st) {
     __shared__ double ss[kGrid], sm[kGrid], sb[kGrid];
-    __shared__ unsigned int sc[kCoarse];
+    __shared__ unsigned int sc[kCoarse + kCoarse / 32];
     __shared__ bool is_last;
     const int tid = threadIdx.x;
     for (int i = tid; i < kCoarse; i += kThreads) sc[i] = 0;
@@ -204,14 +205,16 @@ __global__ void __launch_bounds__(kThreads) k_partials(const double* w, int64_t 
     unsigned long long* sk = reinterpret_cast<unsigned long long*>(sm);
     __shared__ int best;
     auto edge = [](int j) { return __longlong_as_double(static_cast<long long>(j) << kCoarseShift); };
-    for (int i = tid; i < kCoarse; i += kThreads) sc[i] = __ldcg(coarse + i);
+    // (one word of padding per 32: a thread walks its slice of 32 buckets, and unpadded the lanes of a warp shared one bank)
+    auto at = [](int j) { return j + (j >> 5); };
+    for (int i = tid; i < kCoarse; i += kThreads) sc[at(i)] = __ldcg(coarse + i);
     if (tid == 0) best = 0;
     __syncthreads();
     const int lane = tid & 31, warp = tid >> 5;
     double A = 0.0;
     unsigned long long K = 0;
     for (int j = kPer - 1; j >= 0; --j)
-        if (const unsigned int c = sc[tid * kPer + j]) {
+        if (const unsigned int c = sc[at(tid * kPer + j)]) {
             A += static_cast<double>(c) * edge(tid * kPer + j);
             K += c;
         }
@@ -240,7 +243,7 @@ __global__ void __launch_bounds__(kThreads) k_partials(const double* w, int64_t 
     const unsigned long long K_above = K;
     for (int j = kPer - 1; j >= 0; --j) {
         const int b = tid * kPer + j;
-        const unsigned int c = sc[b];
+        const unsigned int c = sc[at(b)];
         if (c == 0) continue;
         const double T = edge(b);
         A += static_cast<double>(c) * T;
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(kThreads) k_partials(const double* w, int64_t 
     // weights at or above the chosen edge
     if (tid == best / kPer) {
         K = K_above;
-        for (int j = kPer - 1; j >= best % kPer; --j) K += sc[tid * kPer + j];
+        for (int j = kPer - 1; j >= best % kPer; --j) K += sc[at(tid * kPer + j)];
         State x{};
         x.S = S;
         x.wmax = wmax;
@@ -345,28 +348,36 @@ __global__ void __launch_bounds__(kThreads) k_pass(const double* w, int64_t n, c
             sc[j / kBuckets][j % kBuckets] = 0;
         }
         __syncthreads();
-        for (int64_t base = b0; base < b1; base += kThreads) {  // block-uniform trip count (warp collectives)
-            const int64_t i = base + tid;
-            const unsigned long long u = i < b1 ? __ldcg(src + i) : ~0ULL;
-            const bool in = valid_bits(u) && u >= lo && u < hi;
-            if (__ballot_sync(0xffffffffu, in) == 0) continue;
-            const int bk = in ? static_cast<int>((u - lo) >> shift) : -1;
-            const unsigned long long v = in ? fixed_units(u, sexp[bk]) : 0ULL;
-            // lanes of one bucket combine first: exact 21-bit limb sums, one leader per bucket
-            const unsigned grp = __match_any_sync(0xffffffffu, bk);
-            const unsigned l0 = __reduce_add_sync(grp, static_cast<unsigned>(v & 0x1FFFFF));
-            const unsigned l1 = __reduce_add_sync(grp, static_cast<unsigned>((v >> 21) & 0x1FFFFF));
-            const unsigned l2 = __reduce_add_sync(grp, static_cast<unsigned>(v >> 42));
-            if (in && lane == __ffs(grp) - 1) {
-                // l0 + l1 2^21 + l2 2^42 in limbs of 32 bits (l2 below 2^16)
-                const unsigned long long t = static_cast<unsigned long long>(l0) + (static_cast<unsigned long long>(l1) << 21);
-                // one leader per bucket in this warp and the histogram private to the warp: plain
-                // read-modify-write, no atomics
-                s0[warp][bk] += t & 0xFFFFFFFFULL;
-                s1[warp][bk] += (t >> 32) + (static_cast<unsigned long long>(l2) << 10);
-                sc[warp][bk] += static_cast<unsigned>(__popc(grp));
+        for (int64_t base = b0; base < b1; base += kPassUnroll * kThreads) {  // block-uniform trip count (warp collectives)
+            unsigned long long us[kPassUnroll];
+#pragma unroll
+            for (int k = 0; k < kPassUnroll; ++k) {
+                const int64_t i = base + k * kThreads + tid;
+                us[k] = i < b1 ? __ldcg(src + i) : ~0ULL;
             }
-            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < kPassUnroll; ++k) {
+                const unsigned long long u = us[k];
+                const bool in = valid_bits(u) && u >= lo && u < hi;
+                if (__ballot_sync(0xffffffffu, in) == 0) continue;
+                const int bk = in ? static_cast<int>((u - lo) >> shift) : -1;
+                const unsigned long long v = in ? fixed_units(u, sexp[bk]) : 0ULL;
+                // lanes of one bucket combine first: exact 21-bit limb sums, one leader per bucket
+                const unsigned grp = __match_any_sync(0xffffffffu, bk);
+                const unsigned l0 = __reduce_add_sync(grp, static_cast<unsigned>(v & 0x1FFFFF));
+                const unsigned l1 = __reduce_add_sync(grp, static_cast<unsigned>((v >> 21) & 0x1FFFFF));
+                const unsigned l2 = __reduce_add_sync(grp, static_cast<unsigned>(v >> 42));
+                if (in && lane == __ffs(grp) - 1) {
+                    // l0 + l1 2^21 + l2 2^42 in limbs of 32 bits (l2 below 2^16)
+                    const unsigned long long t = static_cast<unsigned long long>(l0) + (static_cast<unsigned long long>(l1) << 21);
+                    // one leader per bucket in this warp and the histogram private to the warp: plain
+                    // read-modify-write, no atomics
+                    s0[warp][bk] += t & 0xFFFFFFFFULL;
+                    s1[warp][bk] += (t >> 32) + (static_cast<unsigned long long>(l2) << 10);
+                    sc[warp][bk] += static_cast<unsigned>(__popc(grp));
+                }
+                __syncwarp();
+            }
         }
         __syncthreads();
         unsigned long long t0 = 0, t1 = 0, c = 0;
@@ -666,7 +677,10 @@ int ps_unweight_max(const double* w, int64_t n, double eps, double* result, void
     const unsigned int cap = static_cast<unsigned int>(list_len(n));
     k_partials<<<kGrid, kThreads, 0, st>>>(w, n, eps, part, coarse, cap, state);
     k_gather<<<kGrid, kThreads, 0, st>>>(w, n, state, list, cap);
-    for (int p = 0; p < kPasses; ++p) k_pass<<<kPassGrid, kThreads, 0, st>>>(w, n, list, cap, state, sums);
+    // A long list's tail may outgrow the workspace: the passes then read all weights, with four blocks an SM (1e7 weights,
+    // eps = 0.6: 776 us with two, 532 with four).  A short one's extra blocks only take tickets (1000: 81 and 83 us).
+    const int grid = n < kSampleFrom ? kPassGrid : 2 * kPassGrid;
+    for (int p = 0; p < kPasses; ++p) k_pass<<<grid, kThreads, 0, st>>>(w, n, list, cap, state, sums);
     k_result<<<1, 32, 0, st>>>(state, result);
     ps::count_launches(4 + kPasses);
     return ucheck(cudaGetLastError(), "ps_unweight_max");
