@@ -221,7 +221,7 @@ int signature(const Graph& g, int op, const std::vector<Arg>& a, std::vector<int
 // ===================================================================== compile
 namespace ps {
 
-int compile_graph(const Graph& g, Compiled* out, std::string* err) {
+int compile_graph(const Graph& g, Compiled* out, std::string* err, bool derive) {
     if (!g.outputs_set) { *err = "graph outputs were not set"; return PS_ERR_GRAPH; }
     const int nv = static_cast<int>(g.type.size());
     const int ni = static_cast<int>(g.code.size());
@@ -276,7 +276,7 @@ int compile_graph(const Graph& g, Compiled* out, std::string* err) {
         // A power-law map between constant bounds reads log1p((x_max - x_min)/lo) as a constant of the channel:
         // a seventh argument of the byte-code (about 13 FP64 instructions per event otherwise).
         std::vector<double> derived;
-        if (in.op == PS_OP_INVARIANT_NU && in.args[1].kind == PS_ARG_IMM && in.args[3].kind == PS_ARG_IMM &&
+        if (derive && in.op == PS_OP_INVARIANT_NU && in.args[1].kind == PS_ARG_IMM && in.args[3].kind == PS_ARG_IMM &&
             in.args[4].kind == PS_ARG_IMM) {
             const double M = in.args[1].imm, lo = in.args[3].imm - (M > 0.0 ? M * M : -in.args[5].imm);
             const double L = std::log1p((in.args[4].imm - in.args[3].imm) / lo);
@@ -1177,6 +1177,21 @@ void free_device(ps_program p) {
 
 int64_t tiles_of(int64_t n, int block) { return (n + block - 1) / block; }
 
+constexpr int kVegasBins = 64;
+
+// shared memory of a CTA of the interpreter (the mixed kernel also stages float immediates)
+size_t interpreter_smem(ps_program p) {
+    ps::LaunchParams lp;
+    std::memset(&lp, 0, sizeof lp);
+    lp.block = p->block;
+    lp.smem_code_ints = p->max_code;
+    lp.smem_imm = p->max_imm;
+    lp.smem_grid = p->max_grid;
+    lp.smem_slots = p->max_slots;
+    lp.mixed = p->opt.precision == PS_PRECISION_MIXED ? 1 : 0;
+    return ps::smem_bytes_for(lp);
+}
+
 // CTAs of a map launch.  The interpreter's four an SM become as many as the launch has tiles where all of them fit
 // at once and the caller asked for no number: a second, partly empty round of tiles costs a tile's latency (generate
 // and statistics of 10^5 2->2 events, 782 tiles: 43.7 -> 40.4 us, mixed 36.2 -> 32.2 us; 1.5e5 mixed 37.5 -> 34.4 us;
@@ -1300,44 +1315,58 @@ int ps_program_create(const ps_graph* graphs, int n_ch, const ps_options* opt, i
         delete p;
         return fail(PS_ERR_INVALID_ARGUMENT, "unsupported precision mode");
     }
-    p->ch.resize(n_ch);
+    const bool mixed = p->opt.precision == PS_PRECISION_MIXED;
     std::vector<int32_t> code;
     std::vector<double> imm;
-    for (int c = 0; c < n_ch; ++c) {
-        std::string err;
-        int st = ps::compile_graph(graphs[c]->g, &p->ch[c], &err);
-        if (st != PS_OK) {
-            delete p;
-            return fail(st, "channel " + std::to_string(c) + ": " + err);
+    // The derived constants (the mixed maps have no use for them) are left out where an interpreter's CTA would not fit
+    // with them.
+    for (bool derive : {true, false}) {
+        if (derive && mixed) continue;
+        code.clear();
+        imm.clear();
+        p->ch.assign(n_ch, Compiled());
+        p->code_off.clear();
+        p->imm_off.clear();
+        p->max_code = p->max_imm = p->max_slots = 0;
+        p->max_grid = ps::kTrigDoubles;
+        for (int c = 0; c < n_ch; ++c) {
+            std::string err;
+            int st = ps::compile_graph(graphs[c]->g, &p->ch[c], &err, derive);
+            if (st != PS_OK) {
+                delete p;
+                return fail(st, "channel " + std::to_string(c) + ": " + err);
+            }
+            const Compiled& C = p->ch[c];
+            if (C.n_momenta_out != p->ch[0].n_momenta_out || C.has_x1 != p->ch[0].has_x1 || C.has_alpha != p->ch[0].has_alpha) {
+                delete p;
+                return fail(PS_ERR_GRAPH, "all channels of a program must declare the same outputs");
+            }
+            p->code_off.push_back(static_cast<int>(code.size()));
+            code.insert(code.end(), C.code.begin(), C.code.end());
+            p->imm_off.push_back(static_cast<int>(imm.size()));
+            imm.insert(imm.end(), C.imm.begin(), C.imm.end());
+            p->max_code = std::max(p->max_code, static_cast<int>(C.code.size()));
+            p->max_imm = std::max(p->max_imm, static_cast<int>(C.imm.size()));
+            p->max_slots = std::max(p->max_slots, C.n_slots);
+            if (C.vegas_dims > 0) p->max_grid = std::max(p->max_grid, ps::kTrigDoubles + C.vegas_dims * (2 * kVegasBins + 1));
         }
-        const Compiled& C = p->ch[c];
-        if (C.n_momenta_out != p->ch[0].n_momenta_out || C.has_x1 != p->ch[0].has_x1 || C.has_alpha != p->ch[0].has_alpha) {
-            delete p;
-            return fail(PS_ERR_GRAPH, "all channels of a program must declare the same outputs");
-        }
-        p->code_off.push_back(static_cast<int>(code.size()));
-        code.insert(code.end(), C.code.begin(), C.code.end());
-        p->imm_off.push_back(static_cast<int>(imm.size()));
-        imm.insert(imm.end(), C.imm.begin(), C.imm.end());
-        p->max_code = std::max(p->max_code, static_cast<int>(C.code.size()));
-        p->max_imm = std::max(p->max_imm, static_cast<int>(C.imm.size()));
-        p->max_slots = std::max(p->max_slots, C.n_slots);
+        int limit = 0;
+        if (p->block > 256 || cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
+            interpreter_smem(p) <= static_cast<size_t>(limit))
+            break;
     }
     // default VEGAS grids: identity with 64 bins.  A CTA's staged-grid region holds the azimuth
     // table, then the grid's edges and bin widths.
     int goff = 0, hoff = 0;
-    p->max_grid = ps::kTrigDoubles;
     for (int c = 0; c < n_ch; ++c) {
         p->grid_off.push_back(goff);
         p->hist_off.push_back(hoff);
         int dv = p->ch[c].vegas_dims;
         if (dv > 0) {
-            const int bins = 64;
             for (int j = 0; j < dv; ++j)
-                for (int k = 0; k <= bins; ++k) p->h_grid.push_back(static_cast<double>(k) / bins);
-            goff += dv * (bins + 1);
-            hoff += dv * bins;
-            p->max_grid = std::max(p->max_grid, ps::kTrigDoubles + dv * (2 * bins + 1));
+                for (int k = 0; k <= kVegasBins; ++k) p->h_grid.push_back(static_cast<double>(k) / kVegasBins);
+            goff += dv * (kVegasBins + 1);
+            hoff += dv * kVegasBins;
         }
     }
     p->grid_off.push_back(goff);
@@ -1370,15 +1399,7 @@ int ps_program_create(const ps_graph* graphs, int n_ch, const ps_options* opt, i
     if (st == PS_OK) st = cuda_check(cudaMemset(p->d_stats_mode, 0, sizeof(int32_t)), "memset stats mode");
     if (st != PS_OK) { free_device(p); delete p; return st; }
 
-    ps::LaunchParams lp;
-    std::memset(&lp, 0, sizeof lp);
-    lp.block = p->block;
-    lp.smem_code_ints = p->max_code;
-    lp.smem_imm = p->max_imm;
-    lp.smem_grid = p->max_grid;
-    lp.smem_slots = p->max_slots;
-    lp.mixed = p->opt.precision == PS_PRECISION_MIXED ? 1 : 0;  // the mixed kernel also stages float immediates
-    p->smem = ps::smem_bytes_for(lp);
+    p->smem = interpreter_smem(p);
     std::string err;
     if (p->block <= 256) {  // the interpreter's launch shape (a compiled program never launches it)
         if (p->smem > static_cast<size_t>(prop.sharedMemPerBlockOptin)) {
@@ -1387,7 +1408,7 @@ int ps_program_create(const ps_graph* graphs, int n_ch, const ps_options* opt, i
             return fail(PS_ERR_CAPACITY, "channel needs " + std::to_string(p->smem) + " bytes of shared memory per CTA");
         }
         int per_sm = 0;
-        st = ps::max_ctas_per_sm(p->block, p->smem, p->opt.precision == PS_PRECISION_MIXED, &per_sm, &err);
+        st = ps::max_ctas_per_sm(p->block, p->smem, mixed, &per_sm, &err);
         if (st != PS_OK || per_sm < 1) {
             free_device(p);
             delete p;
@@ -1399,7 +1420,6 @@ int ps_program_create(const ps_graph* graphs, int n_ch, const ps_options* opt, i
     }
     if (p->opt.flags & PS_PROGRAM_JIT) {  // the compiled kernel: VEGAS grid and reduction scratch in shared memory
         // a requested CTA count also caps the compiled kernel's registers so that many CTAs fit
-        const bool mixed = p->opt.precision == PS_PRECISION_MIXED;
         const int min_blocks = ps::jit_min_blocks(p->ch.size(), mixed, p->block, p->opt.ctas_per_sm);
         p->jit_tiles = ps::jit_cta_tiles(p->ch.size(), mixed, p->block, min_blocks, p->max_grid);
         st = ps::jit_prepare(p->ch, p->block, min_blocks, mixed, p->jit_tiles, device, &p->jit_fn, &err);
@@ -1712,7 +1732,7 @@ int ps_jit_check(const ps_graph* graphs, int n_ch, const ps_options* opt, char* 
     std::string err;
     for (int c = 0; c < n_ch; ++c) {
         if (!graphs[c]) return fail(PS_ERR_INVALID_ARGUMENT, "ps_jit_check: null graph");
-        int st = ps::compile_graph(graphs[c]->g, &ch[c], &err);
+        int st = ps::compile_graph(graphs[c]->g, &ch[c], &err, !mixed);
         if (st != PS_OK) return fail(st, "channel " + std::to_string(c) + ": " + err);
     }
     std::vector<char> cubin;

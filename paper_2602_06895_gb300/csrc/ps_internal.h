@@ -56,7 +56,8 @@ struct Compiled {
     bool has_x1 = false, has_x2 = false, has_alpha = false;
 };
 
-int compile_graph(const Graph& g, Compiled* out, std::string* err);
+// derive: constants of the channel (map_nu's logarithm of a constant range) go along as extra arguments
+int compile_graph(const Graph& g, Compiled* out, std::string* err, bool derive);
 
 // ---------------------------------------------------------------- inverse map plan
 // Everything the inverse kernel needs about one channel, flattened on the host from its
