@@ -1,7 +1,6 @@
-"""The VEGAS training histogram over the grids it accepts: odd and even numbers of mapped dimensions, one bin, bin
-counts that are no power of two and on both sides of the kernel's change of thread count, event counts below and
-above its 112 chunks, Philox and explicit points.  The reference adds w^2 in extended precision: the kernel's sums
-carry at most one rounding per event of a bin."""
+"""The VEGAS training histogram over what it is given: odd and even numbers of mapped dimensions, event counts below and
+above its 112 chunks, Philox and explicit points (64 bins: the number that every grid of the library has).  The reference
+adds w^2 in extended precision: the kernel's sums carry at most one rounding per event of a bin."""
 import numpy as np
 import pytest
 
