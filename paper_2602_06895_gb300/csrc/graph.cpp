@@ -282,10 +282,24 @@ int compile_graph(const Graph& g, Compiled* out, std::string* err, bool derive) 
             const double L = std::log1p((in.args[4].imm - in.args[3].imm) / lo);
             if (lo > 0.0 && std::isfinite(L)) derived.push_back(L);
         }
+        // r_to_x1x2 keeps its fourth argument in the byte-code only where log x2 goes nowhere but, with log x1, into
+        // pairs of densities
+        size_t n_args = in.args.size();
+        if (in.op == PS_OP_R_TO_X1X2 && n_args == 4) {
+            const int l1 = in.outs[3], l2 = in.outs[4];
+            bool pairs = std::find(g.out_ids.begin(), g.out_ids.end(), l2) == g.out_ids.end();
+            for (const Instr& u : g.code)
+                for (size_t k = 0; k < u.args.size(); ++k)
+                    if (u.args[k].kind == PS_ARG_VALUE && u.args[k].id == l2)
+                        pairs &= u.op == PS_OP_PDF_POWER && u.args.size() == 6 && k == 5 &&
+                                 u.args[3].kind == PS_ARG_VALUE && u.args[3].id == l1;
+            if (!pairs) n_args = 3;
+        }
         out->code.push_back(in.op);
-        out->code.push_back(static_cast<int32_t>(in.args.size() + derived.size()));
+        out->code.push_back(static_cast<int32_t>(n_args + derived.size()));
         out->code.push_back(static_cast<int32_t>(in.outs.size()));
-        for (auto& a : in.args) out->code.push_back(a.kind == PS_ARG_VALUE ? slot[a.id] : ~imm(a.imm));
+        for (size_t k = 0; k < n_args; ++k)
+            out->code.push_back(in.args[k].kind == PS_ARG_VALUE ? slot[in.args[k].id] : ~imm(in.args[k].imm));
         for (double v : derived) out->code.push_back(~imm(v));
         // In place: vegas and boost_beam read argument k before they write output k and touch no
         // other argument after that, so output k may take the slot of argument k when that

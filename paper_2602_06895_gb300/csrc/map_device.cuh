@@ -465,7 +465,10 @@ __device__ __forceinline__ void exec_op(const int op, const int32_t* a, const in
                 const double iS = Fr::kStatic ? 1.0 / S : fast::rcp(S);
                 const double tau = shat * iS;
                 double L = fast::log(tau);
-                const double l1 = __dmul_rn(r, L), l2 = __dadd_rn(L, -l1);  // log x1, log x2: their sum is log tau again
+                // log x1, log x2: for the pair of densities (the byte-code keeps the fourth argument) L - l1, so that
+                // their sum is log tau again; for any other reader (1 - r) L to half an ulp, also as r nears 1
+                const bool pair = na > 3;
+                const double l1 = __dmul_rn(r, L), l2 = fma(pair ? -1.0 : -r, pair ? l1 : L, L);
                 const double x1 = fast::exp(l1);
                 st(f, o[0], x1);
                 st(f, o[1], fast::div(tau, x1));  // x1 x2 = tau: a division where a second exponential was
