@@ -1390,7 +1390,7 @@ __device__ __forceinline__ void map_tiles(const LaunchParams& lp, Policy& pol, d
         // each half (lane 0 ends with sum w, lane 16 with sum w^2).  The warps' records are joined by four lanes of the
         // first warp, one a record: the two sums in the same instructions, the count and the maximum as integers.
         // (One thread that joined all four in FP64 took 16 FP64 instructions a tile instead of three: compiled
-        // 2->4, 1e7 events, 7.68 -> 7.31 ms, mixed 1529 -> 1439 us.)
+        // 2->4, 1e7 events, 7.68 -> 7.31 ms, mixed 1529 -> 1435 us.)
         const int warp = tid >> 5, lane = tid & 31;
         const unsigned full = 0xffffffffu;
         const int nz = __popc(__ballot_sync(full, (dbits(w) << 1) != 0));  // w != 0 (NaN counts)
