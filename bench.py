@@ -123,8 +123,9 @@ def fp64_peak(ps, torch, local, reps=5):
 
 def fp64_pipe_roofline(instr_per_event, events_per_s, flops_per_event=None):
     """The FP64-pipe roofline object of a kernel: its FP64 arithmetic instructions per event (from
-    ncu) times its events per second (per GPU) against the FP64 issue peak measured in this run
-    (fp64_peak; the derived 629.3 G/s if it was not taken); with flops per event also the flop form
+    ncu) times its events per second (per GPU) against the issue rate of the probe's loop in this run
+    (fp64_peak: 0.84 of the pipe's own rate, which a kernel can pass by a little; the derived 629.3 G/s,
+    that own rate, if it was not taken); with flops per event also the flop form
     against 1.25 TFLOP/s.  Unknown counters give null fields."""
     achieved = None if instr_per_event is None else instr_per_event * events_per_s / 1e9
     peak = _FP64_PEAK["value"] or FP64_PEAK_GINSTR
