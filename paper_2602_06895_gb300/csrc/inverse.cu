@@ -33,10 +33,11 @@ constexpr int kMaxLeg = kMaxOutMomenta + 2;
 namespace fast = dev::fast;
 
 // Both inverse maps: where rounding has collapsed the range to a point every r maps to it, and 0 is
-// returned (the quotients below would be 0/0 or infinite).
+// returned (the quotients below would be 0/0 or infinite); for a NaN x or NaN bounds, NaN as from the quotients.
 // (comparisons on the bits here and below: the FP64 pipe that bounds the kernel would execute them)
-__device__ __forceinline__ bool empty_range(double xmin, double xmax) {  // x_max <= x_min for bounds >= 0
-    return dev::dbits(xmax) <= dev::dbits(xmin);
+__device__ __forceinline__ bool nan_bits(double v) { return (dev::dbits(v) & 0x7FFFFFFFFFFFFFFFLL) > dev::kInfBits; }
+__device__ __forceinline__ bool empty_range(double x, double xmin, double xmax) {  // x_max <= x_min for bounds >= 0
+    return dev::dbits(xmax) <= dev::dbits(xmin) && !nan_bits(x) && !nan_bits(xmin) && !nan_bits(xmax);
 }
 
 // inverse power-law map (anchored as the forward map; by roots where 1/(1 - nu) is an integer, as there: 31 FP64
@@ -44,7 +45,7 @@ __device__ __forceinline__ bool empty_range(double xmin, double xmax) {  // x_ma
 __device__ __forceinline__ double inv_nu(double x, double m, double nu, double xmin, double xmax, double a) {
     const double m2 = dev::pos_bits(m) ? m * m : -a;
     const double lo = xmin - m2, hi = xmax - m2;
-    if (empty_range(xmin, xmax)) return 0.0;
+    if (empty_range(x, xmin, xmax)) return 0.0;
     const double p = fast::div(xmax - xmin, lo), q = fast::div(x - xmin, lo);
     if (dev::dbits(nu) == dev::dbits(1.0)) return fast::div(fast::log1p(q), fast::log1p(p));
     const double w = 1.0 - nu;
@@ -62,7 +63,7 @@ __device__ __forceinline__ double inv_nu(double x, double m, double nu, double x
 __device__ __forceinline__ double inv_bw(double x, double M, double G, double xmin, double xmax) {
     const double mg = M * G, m2 = M * M;
     const double a = (xmin - m2) / mg, b = (xmax - m2) / mg;
-    if (empty_range(xmin, xmax)) return 0.0;
+    if (empty_range(x, xmin, xmax)) return 0.0;
     const double D = atan2((xmax - xmin) / mg, fma(a, b, 1.0));
     const double t = (x - m2) / mg;
     if (x - xmin <= xmax - x) return atan2((x - xmin) / mg, fma(a, t, 1.0)) / D;
