@@ -683,13 +683,19 @@ int ps_unweight_max(const double* w, int64_t n, double eps, double* result, void
     k_zero<<<(kCoarse + 255) / 256, 256, 0, st>>>(state, coarse, sums);
     const unsigned int cap = static_cast<unsigned int>(list_len(n));
     k_partials<<<kGrid, kThreads, 0, st>>>(w, n, eps, part, coarse, cap, state);
-    k_gather<<<kGrid, kThreads, 0, st>>>(w, n, state, list, cap);
-    // A long list's tail may outgrow the workspace: the passes then read all weights, with four blocks an SM (1e7 weights,
-    // eps = 0.6: 776 us with two, 532 with four).  A short one's extra blocks only take tickets (1000: 81 and 83 us).
-    const int grid = n < kSampleFrom ? kPassGrid : 2 * kPassGrid;
-    for (int p = 0; p < kPasses; ++p) k_pass<<<grid, kThreads, 0, st>>>(w, n, list, cap, state, sums);
+    int launches = 3;
+    // eps = 0 is the maximum itself, which k_partials has: no search (1e5 weights: 70 us with the search's launches, 65 before
+    // there was a list, 28 now)
+    if (eps > 0.0) {
+        k_gather<<<kGrid, kThreads, 0, st>>>(w, n, state, list, cap);
+        // A long list's tail may outgrow the workspace: the passes then read all weights, with four blocks an SM (1e7
+        // weights, eps = 0.6: 776 us with two, 532 with four).  A short one's extra blocks only take tickets (1000: 81 and 83 us).
+        const int grid = n < kSampleFrom ? kPassGrid : 2 * kPassGrid;
+        for (int p = 0; p < kPasses; ++p) k_pass<<<grid, kThreads, 0, st>>>(w, n, list, cap, state, sums);
+        launches += 1 + kPasses;
+    }
     k_result<<<1, 32, 0, st>>>(state, result);
-    ps::count_launches(4 + kPasses);
+    ps::count_launches(launches);
     return ucheck(cudaGetLastError(), "ps_unweight_max");
 }
 
